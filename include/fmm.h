@@ -59,7 +59,10 @@ typedef enum {
 } fmm_status_t;
 
 typedef enum {
-    FMM_PREC_FP32 = 0,   /* 3 x TF32: hi*hi + hi*lo + lo*hi, fp32 accumulate (FP32-class) */
+    FMM_PREC_FP32 = 0,   /* hi*hi + hi*lo + lo*hi of TF32 hi parts, fp32 accumulate (FP32-class):
+                            three TF32 products, or, on CTA-pair leaves of a range of lengths
+                            at depths 0 to 2 where its total error is the smaller, one TF32
+                            product and the two corrections in bf16 */
     FMM_PREC_TF32 = 1,   /* one TF32 product, fp32 accumulate */
     FMM_PREC_BF16X3 = 2, /* bfloat16 hi/lo split, 3 products, fp32 accumulate */
     FMM_PREC_FP16X3 = 3  /* IEEE half hi/lo split with power-of-two scaling, 3 products */

@@ -476,8 +476,39 @@ __global__ void __launch_bounds__(128) quad_post_kernel(QuadPost q) {
 // The planes are written with evict-first (streaming) stores: they are read by
 // the leaf launch only after far more data than L2 holds has passed, and they
 // must not push out the operand lines a fused pass reads again.
+//   tf32x:       hi = rn_tf32(x) (trunc_tf32(x) where the leaves read the raw operand), and in the
+//                other plane bf16(hi) and bf16(x - hi), 32 columns of each per 128-byte line
+// Nearest TF32 value (ties away from zero); what would round past the largest
+// finite value, and infinities, keep their truncation.
+__device__ __forceinline__ float tf32x_hi(float x) {
+    const uint32_t u = __float_as_uint(x), r = (u + 0x1000u) & 0xFFFFE000u;
+    return __uint_as_float((r & 0x7F800000u) == 0x7F800000u ? (u & 0xFFFFE000u) : r);
+}
+// Two values to bf16, nearest even, saturating at the largest finite value.
+__device__ __forceinline__ uint32_t bf16x2_sat(float x0, float x1) {
+    uint32_t r;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(x1), "f"(x0));
+    return r;
+}
+// 16-bit offset of hi (lo: + 32) of the element at offset o of a tf32x correction plane.
+__device__ __forceinline__ long long tf32x_off(long long o) { return 2 * (o & ~31LL) + (o & 31); }
+
 template <int KIND>
 __device__ __forceinline__ void split_store(void* hi_plane, void* lo_plane, long long o, float4 v, float sc) {
+    if constexpr (KIND == kSplitTF32X) {
+        float4 h;
+        if (hi_plane) {
+            h = f4(tf32x_hi(v.x), tf32x_hi(v.y), tf32x_hi(v.z), tf32x_hi(v.w));
+            __stcs(reinterpret_cast<float4*>(static_cast<float*>(hi_plane) + o), h);
+        } else {
+            h = f4(tf32_trunc(v.x), tf32_trunc(v.y), tf32_trunc(v.z), tf32_trunc(v.w));
+        }
+        uint16_t* hl = static_cast<uint16_t*>(lo_plane) + tf32x_off(o);
+        __stcs(reinterpret_cast<uint2*>(hl), make_uint2(bf16x2_sat(h.x, h.y), bf16x2_sat(h.z, h.w)));
+        __stcs(reinterpret_cast<uint2*>(hl + 32),
+               make_uint2(bf16x2_sat(v.x - h.x, v.y - h.y), bf16x2_sat(v.z - h.z, v.w - h.w)));
+        return;
+    }
     if constexpr (KIND == kSplitTF32) {
         float4 l;
         l.x = tf32_round_rne(v.x - tf32_trunc(v.x));
@@ -510,14 +541,22 @@ __device__ __forceinline__ void split_store(void* hi_plane, void* lo_plane, long
     __stcs(reinterpret_cast<uint2*>(lo), make_uint2(l01, l23));
 }
 
+// Columns a split pass writes of a matrix of `cols` columns: a tf32x correction
+// plane is zero up to the next multiple of 32 (the planes' pitch covers it).
+template <int KIND>
+__host__ __device__ __forceinline__ long long plane_cols(long long cols) {
+    return KIND == kSplitTF32X ? (cols + 31) & ~31LL : cols;
+}
+
 // Same arithmetic as pre_add_kernel (all 7 children), output split into planes.
 template <bool VEC, int SIDE_B, int KIND>
 __global__ void __launch_bounds__(128) pre_add16_kernel(View P, long long h, long long w, Stack16 out,
                                                         const float* __restrict__ scale) {
     const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-    if (c >= w) return;
+    if (c >= plane_cols<KIND>(w)) return;
     const float sc = scale ? scale[SIDE_B] : 1.0f;
     const long long node = blockIdx.z;
+    if (c >= w) P.valid_rows = 0;   // padding columns of a tf32x plane: zeros
     const float* base = P.ptr + node * P.node_stride;
     const float* q1p = base + w;
     const float* q2p = base + h * P.ld;
@@ -575,7 +614,7 @@ __global__ void __launch_bounds__(256) pre_add16_b_root_kernel(const float* __re
     const int t = ty * 32 + tx;          // 0..255
     const int nl = t >> 3, kq = (t & 7) * 4;
     const long long n = n0 + nl, k = k0 + kq;
-    if (n < nh && k < kh) {
+    if (n < nh && k < plane_cols<KIND>(kh)) {
 #pragma unroll
         for (int c = 0; c < 7; ++c) {
             const float4 v = make_float4(tile[c][kq][nl], tile[c][kq + 1][nl], tile[c][kq + 2][nl], tile[c][kq + 3][nl]);
@@ -621,7 +660,7 @@ __global__ void __launch_bounds__(256) split16_kernel(const float* __restrict__ 
             const int g = tid + 256 * j;
             const long long r = r0 + (g >> 5), c = c0 + 4 * (g & 31);
             // ld is a multiple of 8, so a group of 4 never crosses a row: padding columns get zeros
-            if (r < rows && c < cols) split_store<KIND>(out.hi, out.lo, r * out.ld + c, v[j], sc);
+            if (r < rows && c < plane_cols<KIND>(cols)) split_store<KIND>(out.hi, out.lo, r * out.ld + c, v[j], sc);
         }
         return;
     }
@@ -641,7 +680,7 @@ __global__ void __launch_bounds__(256) split16_kernel(const float* __restrict__ 
         const int g = tid + 256 * j;   // plane row g / 32 (a column of X), 4 consecutive plane columns
         const int a = g >> 5, q = (g & 31) * 4;
         const long long orow = c0 + a, ocol = r0 + q;
-        if (orow < cols && ocol < rows) {
+        if (orow < cols && ocol < plane_cols<KIND>(rows)) {
             const float4 v = make_float4(tile[a][q], tile[a][q + 1], tile[a][q + 2], tile[a][q + 3]);
             split_store<KIND>(out.hi, out.lo, orow * out.ld + ocol, v, sc);
         }
@@ -684,7 +723,8 @@ template <bool VEC, int SIDE_B, int KIND>
 __global__ void __launch_bounds__(128) pre_add2_kernel(View P, long long h, long long w, Stack16 out,
                                                        const float* __restrict__ scale) {
     const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-    if (c >= w) return;
+    if (c >= plane_cols<KIND>(w)) return;
+    if (c >= w) P.valid_rows = 0;   // padding columns of a tf32x plane: zeros
     const float sc = scale ? scale[SIDE_B] : 1.0f;
     const long long node = blockIdx.z;
     const float* base = P.ptr + node * P.node_stride;
@@ -748,6 +788,15 @@ __device__ __forceinline__ float child_of1(int i, float Q0, float Q1, float Q2, 
 // One value into the planes at element offset o (evict-first stores).
 template <int KIND>
 __device__ __forceinline__ void split_store1(void* hi_plane, void* lo_plane, long long o, float v, float sc) {
+    if constexpr (KIND == kSplitTF32X) {
+        const float hv = tf32x_hi(v);
+        const uint32_t p = bf16x2_sat(hv, v - hv);
+        unsigned short* hl = static_cast<unsigned short*>(lo_plane) + tf32x_off(o);
+        __stcs(static_cast<float*>(hi_plane) + o, hv);
+        __stcs(hl, (unsigned short)(p & 0xffffu));
+        __stcs(hl + 32, (unsigned short)(p >> 16));
+        return;
+    }
     if constexpr (KIND == kSplitTF32) {
         __stcs(static_cast<float*>(hi_plane) + o, v);
         __stcs(static_cast<float*>(lo_plane) + o, tf32_round_rne(v - tf32_trunc(v)));
@@ -782,7 +831,8 @@ template <int SIDE_B, int KIND>
 __global__ void __launch_bounds__(256, 2) pre_add3_kernel(View P, long long h, long long w, Stack16 out,
                                                        const float* __restrict__ scale) {
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= w) return;
+    if (c >= plane_cols<KIND>(w)) return;
+    if (c >= w) P.valid_rows = 0;   // padding columns of a tf32x plane: zeros
     const float sc = scale ? scale[SIDE_B] : 1.0f;
     const long long node = blockIdx.z;
     const float* base = P.ptr + node * P.node_stride;
@@ -873,7 +923,7 @@ __global__ void __launch_bounds__(256, 2) pre_add3_bt_kernel(const float* __rest
     __syncthreads();
     const int tn = t >> 5, tk = t & 31;
     const long long n = n0 + tn, k = k0 + tk;
-    if (n >= h || k >= w) return;
+    if (n >= h || k >= plane_cols<KIND>(w)) return;
     float X[8][8];   // sub-block (a, b) of B^T at position (n, k)
 #pragma unroll
     for (int a = 0; a < 8; ++a)
@@ -935,7 +985,7 @@ __global__ void __launch_bounds__(256) pre_add2_b_root_kernel(const float* __res
     const int t = ty * 32 + tx;
     const int nl = t >> 3, kq = (t & 7) * 4;   // store role: 4 consecutive k of row n0 + nl
     const long long on = n0 + nl, ok = k0 + kq;
-    const bool store = on < h && ok < w;
+    const bool store = on < h && ok < plane_cols<KIND>(w);
 #pragma unroll 1
     for (int i = 0; i < 7; ++i) {
         float4 Ci[4];   // child i's quadrant t
@@ -1117,6 +1167,8 @@ __global__ void __launch_bounds__(128, 4) post_add3_kernel(const float* __restri
 // 16-byte loads to the planes (a warp covers 512 contiguous bytes of a row);
 // transposed jobs stage the block in a 32 x 129 shared tile (conflict-free both
 // ways) and leave it as 128 rows of 32 elements.
+//
+// KIND tf32x: jobs of both FP32 plane forms, by SplitJob::corr16.
 template <int KIND>
 __global__ void __launch_bounds__(256) batched_split_kernel(const SplitJob* __restrict__ jobs, int njobs) {
     __shared__ float tile[32][129];
@@ -1155,7 +1207,11 @@ __global__ void __launch_bounds__(256) batched_split_kernel(const SplitJob* __re
             const int g = tid + 256 * j;
             const long long r = r0 + (g >> 5), c = c0 + 4 * (g & 31);
             // ld is a multiple of 8, so a group of 4 never crosses a row: padding columns get zeros
-            if (r < J.rows && c < J.cols) split_store<KIND>(J.dst, J.lo, r * J.ldd + c, v[j], sc);
+            if (KIND == kSplitTF32X && !J.corr16) {
+                if (r < J.rows && c < J.cols) split_store<kSplitTF32>(J.dst, J.lo, r * J.ldd + c, v[j], sc);
+            } else if (r < J.rows && c < plane_cols<KIND>(J.cols)) {
+                split_store<KIND>(J.dst, J.lo, r * J.ldd + c, v[j], sc);
+            }
         }
         return;
     }
@@ -1179,9 +1235,13 @@ __global__ void __launch_bounds__(256) batched_split_kernel(const SplitJob* __re
         const int g = tid + 256 * j;   // output row a (a source column), 4 consecutive output columns
         const int a = g >> 3, q = (g & 7) * 4;
         const long long orow = c0 + a, ocol = r0 + q;
-        if (orow < J.cols && ocol < J.rows) {
+        if (orow < J.cols && ocol < plane_cols<KIND>(J.rows)) {
             const float4 v = make_float4(tile[q][a], tile[q + 1][a], tile[q + 2][a], tile[q + 3][a]);
-            split_store<KIND>(J.dst, J.lo, orow * J.ldd + ocol, v, sc);
+            if (KIND == kSplitTF32X && !J.corr16) {
+                if (ocol < J.rows) split_store<kSplitTF32>(J.dst, J.lo, orow * J.ldd + ocol, v, sc);
+            } else {
+                split_store<KIND>(J.dst, J.lo, orow * J.ldd + ocol, v, sc);
+            }
         }
     }
 }
@@ -1305,6 +1365,7 @@ cudaError_t launch_pre_add16(const View& parent, long long nodes, const Stack16&
     switch (kind) {                                                          \
         case kSplitBF16: FMM_PRE16(V, S, kSplitBF16); break;                \
         case kSplitFP16: FMM_PRE16(V, S, kSplitFP16); break;                \
+        case kSplitTF32X: FMM_PRE16(V, S, kSplitTF32X); break;              \
         default: FMM_PRE16(V, S, kSplitTF32); break;                        \
     }
     if (vec) { if (side_b) { FMM_PRE16K(true, 1) } else { FMM_PRE16K(true, 0) } }
@@ -1326,6 +1387,9 @@ cudaError_t launch_pre_add16_b_root(const float* B, long long ldb, long long K, 
         case kSplitFP16:
             pre_add16_b_root_kernel<kSplitFP16><<<grid, dim3(32, 8), 0, stream>>>(B, ldb, K, N, kh, nh, out, scale);
             break;
+        case kSplitTF32X:
+            pre_add16_b_root_kernel<kSplitTF32X><<<grid, dim3(32, 8), 0, stream>>>(B, ldb, K, N, kh, nh, out, scale);
+            break;
         default:
             pre_add16_b_root_kernel<kSplitTF32><<<grid, dim3(32, 8), 0, stream>>>(B, ldb, K, N, kh, nh, out, scale);
     }
@@ -1343,6 +1407,7 @@ cudaError_t launch_split16(const float* X, long long ldx, long long rows, long l
     switch (kind) {                                      \
         case kSplitBF16: FMM_SPLIT(kSplitBF16, T); break; \
         case kSplitFP16: FMM_SPLIT(kSplitFP16, T); break; \
+        case kSplitTF32X: FMM_SPLIT(kSplitTF32X, T); break; \
         default: FMM_SPLIT(kSplitTF32, T); break;         \
     }
     if (transpose) { FMM_SPLITK(true) } else { FMM_SPLITK(false) }
@@ -1363,6 +1428,7 @@ cudaError_t launch_pre_add2(const View& node, long long nodes, const Stack16& ou
     switch (kind) {                                             \
         case kSplitBF16: FMM_PRE2(V, S, kSplitBF16); break;    \
         case kSplitFP16: FMM_PRE2(V, S, kSplitFP16); break;    \
+        case kSplitTF32X: FMM_PRE2(V, S, kSplitTF32X); break;  \
         default: FMM_PRE2(V, S, kSplitTF32); break;            \
     }
     if (vec) { if (side_b) { FMM_PRE2K(true, 1) } else { FMM_PRE2K(true, 0) } }
@@ -1381,6 +1447,7 @@ cudaError_t launch_pre_add2_b_root(const float* B, long long ldb, long long K, l
     switch (kind) {
         case kSplitBF16: pre_add2_b_root_kernel<kSplitBF16><<<grid, block, 0, stream>>>(B, ldb, K, N, h, w, out, scale); break;
         case kSplitFP16: pre_add2_b_root_kernel<kSplitFP16><<<grid, block, 0, stream>>>(B, ldb, K, N, h, w, out, scale); break;
+        case kSplitTF32X: pre_add2_b_root_kernel<kSplitTF32X><<<grid, block, 0, stream>>>(B, ldb, K, N, h, w, out, scale); break;
         default: pre_add2_b_root_kernel<kSplitTF32><<<grid, block, 0, stream>>>(B, ldb, K, N, h, w, out, scale); break;
     }
     return cudaGetLastError();
@@ -1396,6 +1463,7 @@ cudaError_t launch_pre_add3(const View& node, long long nodes, const Stack16& ou
     switch (kind) {                                          \
         case kSplitBF16: FMM_PRE3(S, kSplitBF16); break;    \
         case kSplitFP16: FMM_PRE3(S, kSplitFP16); break;    \
+        case kSplitTF32X: FMM_PRE3(S, kSplitTF32X); break;  \
         default: FMM_PRE3(S, kSplitTF32); break;            \
     }
     if (side_b) { FMM_PRE3K(1) } else { FMM_PRE3K(0) }
@@ -1430,6 +1498,7 @@ cudaError_t launch_pre_add3_bt(const float* B, long long ldb, long long K, long 
     switch (kind) {
         case kSplitBF16: return launch_pre_add3_bt_impl<kSplitBF16>(B, ldb, K, N, h, w, out, scale, stream);
         case kSplitFP16: return launch_pre_add3_bt_impl<kSplitFP16>(B, ldb, K, N, h, w, out, scale, stream);
+        case kSplitTF32X: return launch_pre_add3_bt_impl<kSplitTF32X>(B, ldb, K, N, h, w, out, scale, stream);
         default: return launch_pre_add3_bt_impl<kSplitTF32>(B, ldb, K, N, h, w, out, scale, stream);
     }
 }
@@ -1470,6 +1539,7 @@ cudaError_t launch_batched_split(const SplitJob* jobs, int njobs, long long tota
     switch (kind) {
         case kSplitBF16: batched_split_kernel<kSplitBF16><<<(unsigned)total_tiles, dim3(32, 8), 0, stream>>>(jobs, njobs); break;
         case kSplitFP16: batched_split_kernel<kSplitFP16><<<(unsigned)total_tiles, dim3(32, 8), 0, stream>>>(jobs, njobs); break;
+        case kSplitTF32X: batched_split_kernel<kSplitTF32X><<<(unsigned)total_tiles, dim3(32, 8), 0, stream>>>(jobs, njobs); break;
         default: batched_split_kernel<kSplitTF32><<<(unsigned)total_tiles, dim3(32, 8), 0, stream>>>(jobs, njobs);
     }
     return cudaGetLastError();

@@ -126,13 +126,13 @@ fmm_status_t encode_map(CUtensorMap* map, const float* base, long long cols, lon
 fmm_status_t encode_map16(CUtensorMap* map, const void* base, int kind, long long cols, long long rows,
                           long long batch, long long ld, long long batch_stride, int box_rows, bool wide = false) {
     if (cols <= 0 || rows <= 0 || batch <= 0) return FMM_ERR_INVALID_ARG;
-    const long long es = kind == kSplitTF32 ? 4 : 2;
+    const long long es = split_is32(kind) ? 4 : 2;
     if ((reinterpret_cast<uintptr_t>(base) & 15) || (ld * es) % 16 || (batch_stride * es) % 16) return FMM_ERR_ALIGNMENT;
     cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)batch};
     cuuint64_t strides[2] = {(cuuint64_t)(ld * es), (cuuint64_t)(batch_stride * es)};
     cuuint32_t box[3] = {(cuuint32_t)((wide ? 128 : 64) / es), (cuuint32_t)box_rows, 1u};
     cuuint32_t estr[3] = {1u, 1u, 1u};
-    const CUtensorMapDataType dt = kind == kSplitTF32   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+    const CUtensorMapDataType dt = split_is32(kind)     ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                    : kind == kSplitBF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
                                                         : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
     CUresult r = g_encode(map, dt, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -186,7 +186,9 @@ struct fmm_plan_s {
     void* a16[2] = {};   // hi, lo planes of the leaf A operands (stack or the whole A)
     void* b16[2] = {};   // hi, lo planes of the leaf B^T operands
     long long ld16 = 0;
-    size_t es16() const { return split_kind == kSplitTF32 ? 4 : 2; }
+    size_t es16() const { return split_is32(split_kind) ? 4 : 2; }
+    // columns of the lo (correction) plane's tensor map for k columns of an operand
+    long long lo_cols(long long k) const { return split_kind == kSplitTF32X ? (k + 31) / 32 * 32 : k; }
     // depth >= 4: the last three levels of pre-additions (split-plane plans) and
     // of post-additions run as one pass each; the middle levels are never stored
     bool fuse_pre() const { return pre16 && depth >= 4; }
@@ -412,6 +414,31 @@ int leaf_mode(fmm_precision_t p) {
     }
 }
 
+// Columns of a leaf's operands at depth d (padded, or the peeled core's).
+long long leaf_k(long long K, int d, bool peel) {
+    if (d == 0) return K;
+    const long long g = 4LL << d;
+    return (peel ? K / g * g : rup(K, g)) >> d;
+}
+
+// Whether FP32 leaves of k columns at this depth, on CTA pairs, take the TF32
+// product with bf16 corrections (kSplitTF32X) instead of three TF32 products.
+// Their operands carry about 2^-20.7 of rounding (three TF32 products: 2^-23),
+// but the truncating accumulator, 1.9e-8 per instruction and leaf, gets two
+// instructions per 16 columns of K fewer.  From the lower limits on the sum of
+// both is no larger than with three TF32 products (depth 0: equal near K = 150;
+// a level amplifies the operands' part by 2.6, the accumulator's hardly).  Up to
+// the upper limits the two results agree within 2e-5 in the 2-norm (depth 0,
+// K = 4096: 1.0e-5; depth 2, K = 2048: 1.03e-5; depth 3, K = 2048: 2.4e-5, not taken).
+bool tf32x_leaf(long long k, int depth) {
+    switch (depth) {
+        case 0: return k >= 192 && k <= 6144;
+        case 1: return k >= 512 && k <= 6144;
+        case 2: return k >= 1024 && k <= 3072;
+        default: return false;
+    }
+}
+
 // Whether plans that can fuse the last Winograd level into the leaf launch do
 // so when the caller leaves fmm_options_t.fuse_last at 0.
 constexpr bool kFuseLastDefault = true;
@@ -550,7 +577,7 @@ fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const flo
     long long lda = p->lda;
     // FP32 (3xTF32): the hi plane is the raw value, so an aligned A is read in
     // place and only its lo plane is written
-    const bool a_raw = p->pre16 && bf == kSplitTF32 && (reinterpret_cast<uintptr_t>(A) & 15) == 0 && p->lda % 4 == 0;
+    const bool a_raw = p->pre16 && split_is32(bf) && (reinterpret_cast<uintptr_t>(A) & 15) == 0 && p->lda % 4 == 0;
     if (p->pre16) {
         const float* scale = p->mode == kLeafFP16x3P ? p->fp16_scale() : nullptr;
         Stack16 sa{a_raw ? nullptr : p->a16[0], p->a16[1], ld, 0, 1};
@@ -586,11 +613,12 @@ fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const flo
                     if ((s = encode_map16(&args.maps[0], A + k0, bf, kc, p->M, 1, p->lda, p->M * p->lda, kBM,
                                           p->pair)) != FMM_OK)
                         return s;
-                } else if ((s = encode_map16(&args.maps[i], static_cast<char*>(p->a16[i]) + off, bf, kc, p->M, 1, ld,
-                                             p->M * ld, kBM, p->pair)) != FMM_OK) {
+                } else if ((s = encode_map16(&args.maps[i], static_cast<char*>(p->a16[i]) + off, bf,
+                                             i ? p->lo_cols(kc) : kc, p->M, 1, ld, p->M * ld, kBM, p->pair)) != FMM_OK) {
                     return s;
                 }
-                if ((s = encode_map16(&args.maps[2 + i], static_cast<char*>(p->b16[i]) + off, bf, kc, p->N, 1, ld,
+                if ((s = encode_map16(&args.maps[2 + i], static_cast<char*>(p->b16[i]) + off, bf,
+                                      i ? p->lo_cols(kc) : kc, p->N, 1, ld,
                                       p->N * ld, p->pair ? 128 : p->bn, p->pair)) != FMM_OK)
                     return s;
             }
@@ -606,6 +634,7 @@ fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const flo
         G.C = C; G.ldc = p->ldc; G.c_batch_stride = 0;
         G.alpha = alpha; G.beta = first ? beta : 1.0f;
         G.vec_ok = ((reinterpret_cast<uintptr_t>(C) & 15) == 0 && p->ldc % 4 == 0) ? 1 : 0;
+        G.corr16 = p->split_kind == kSplitTF32X ? 1 : 0;
         args.num_groups = 1;
         if ((s = run_leaves(p, args, stream)) != FMM_OK) return s;
         if (!first) p->acct[1] += 8.0 * (double)(p->M * p->N);   // the accumulating launch reads and writes C
@@ -773,11 +802,11 @@ fmm_status_t winograd_leaf_groups(fmm_plan_s* p, CUtensorMap* maps, int& nm, Gem
         const long long batch = Lf.nodes, ld = p->ld16;
         const int bf = p->split_kind;
         for (int i = 0; i < 2; ++i) {
-            if ((s = encode_map16(&maps[nm + i], p->a16[i], bf, kk, mm, batch, ld, mm * ld, kBM, p->pair)) != FMM_OK)
+            const long long cols = i ? p->lo_cols(kk) : kk;
+            if ((s = encode_map16(&maps[nm + i], p->a16[i], bf, cols, mm, batch, ld, mm * ld, kBM, p->pair)) != FMM_OK)
                 return s;
-            if ((s = encode_map16(&maps[nm + 2 + i], p->b16[i], bf, kk, nn, batch, ld, nn * ld, p->pair ? 128 : p->bn,
-                                  p->pair)) !=
-                FMM_OK)
+            if ((s = encode_map16(&maps[nm + 2 + i], p->b16[i], bf, cols, nn, batch, ld, nn * ld,
+                                  p->pair ? 128 : p->bn, p->pair)) != FMM_OK)
                 return s;
         }
         GemmGroup& G = groups[ng++];
@@ -792,6 +821,7 @@ fmm_status_t winograd_leaf_groups(fmm_plan_s* p, CUtensorMap* maps, int& nm, Gem
         }
         G.alpha = 1.f; G.beta = 0.f; G.map_a = nm; G.map_a_lo = nm + 1; G.map_b = nm + 2; G.map_b_lo = nm + 3;
         G.vec_ok = 1;
+        G.corr16 = p->split_kind == kSplitTF32X ? 1 : 0;
         nm += 4;
         return FMM_OK;
     }
@@ -1034,10 +1064,14 @@ fmm_status_t batched_build(fmm_batched_s* b, int count, const int64_t* M, const 
     b->bn = (lt && lt != 512) ? lt : 256;
     b->tile = b->pair ? 512 : b->bn;
     if (b->pre) {
-        b->split_kind = o.precision == FMM_PREC_BF16X3 ? kSplitBF16 : b->fp16 ? kSplitFP16 : kSplitTF32;
+        // kSplitTF32X: each problem takes one of the two FP32 plane forms
+        b->split_kind = o.precision == FMM_PREC_BF16X3 ? kSplitBF16
+                        : b->fp16                      ? kSplitFP16
+                        : b->pair                      ? kSplitTF32X
+                                                       : kSplitTF32;
         b->mode = o.precision == FMM_PREC_BF16X3 ? kLeafBF16x3P : b->fp16 ? kLeafFP16x3P : kLeaf3xTF32P;
     }
-    const size_t es = b->split_kind == kSplitTF32 ? 4 : 2;
+    const size_t es = split_is32(b->split_kind) ? 4 : 2;
     // per-problem depth and resource counts
     int total_maps = 0, total_groups = 0, total_jobs = 0;
     b->depth.assign(count, 0);
@@ -1090,24 +1124,27 @@ fmm_status_t batched_build(fmm_batched_s* b, int count, const int64_t* M, const 
             if (!ws) continue;
             // FP32 (3xTF32) planes hold the raw value as hi: an aligned A is read in place
             // and only its lo plane is written
-            const bool a_raw = b->split_kind == kSplitTF32 && (reinterpret_cast<uintptr_t>(A[i]) & 15) == 0 &&
+            const bool a_raw = split_is32(b->split_kind) && (reinterpret_cast<uintptr_t>(A[i]) & 15) == 0 &&
                                lda[i] % 4 == 0;
-            sjobs.push_back(SplitJob{A[i], lda[i], M[i], K[i], a_raw ? nullptr : ah, al, ld, 0,
-                                     (int)((K[i] + 127) / 128), 0, scale_of(i)});
-            sjobs.push_back(SplitJob{B[i], ldb[i], K[i], N[i], bh, bl, ld, 0, (int)((N[i] + 127) / 128), 1, scale_of(i)});
-            fmm_status_t s;
             const int kd = b->split_kind;
+            const int corr16 = kd == kSplitTF32X && tf32x_leaf(K[i], 0) ? 1 : 0;
+            const long long klo = corr16 ? rup(K[i], 32) : K[i];   // columns of the lo / correction plane
             const bool wide = b->pair != 0;              // pair: 128-byte rows, 128 rows of B per CTA
             const int bbox = wide ? 128 : b->bn;
+            sjobs.push_back(SplitJob{A[i], lda[i], M[i], K[i], a_raw ? nullptr : ah, al, ld, 0,
+                                     (int)((K[i] + 127) / 128), 0, scale_of(i), corr16});
+            sjobs.push_back(SplitJob{B[i], ldb[i], K[i], N[i], bh, bl, ld, 0, (int)((N[i] + 127) / 128), 1, scale_of(i),
+                                     corr16});
+            fmm_status_t s;
             if (a_raw) {
                 if ((s = encode_map16(&maps[nm], A[i], kd, K[i], M[i], 1, lda[i], M[i] * lda[i], kBM, wide)) != FMM_OK)
                     return s;
             } else if ((s = encode_map16(&maps[nm], ah, kd, K[i], M[i], 1, ld, M[i] * ld, kBM, wide)) != FMM_OK) {
                 return s;
             }
-            if ((s = encode_map16(&maps[nm + 1], al, kd, K[i], M[i], 1, ld, M[i] * ld, kBM, wide)) != FMM_OK) return s;
+            if ((s = encode_map16(&maps[nm + 1], al, kd, klo, M[i], 1, ld, M[i] * ld, kBM, wide)) != FMM_OK) return s;
             if ((s = encode_map16(&maps[nm + 2], bh, kd, K[i], N[i], 1, ld, N[i] * ld, bbox, wide)) != FMM_OK) return s;
-            if ((s = encode_map16(&maps[nm + 3], bl, kd, K[i], N[i], 1, ld, N[i] * ld, bbox, wide)) != FMM_OK) return s;
+            if ((s = encode_map16(&maps[nm + 3], bl, kd, klo, N[i], 1, ld, N[i] * ld, bbox, wide)) != FMM_OK) return s;
             GemmGroup& G = groups[ng++];
             memset(&G, 0, sizeof(G));
             G.M = (int)M[i]; G.N = (int)N[i]; G.K = (int)K[i]; G.batch = 1;
@@ -1115,6 +1152,7 @@ fmm_status_t batched_build(fmm_batched_s* b, int count, const int64_t* M, const 
             G.map_a = nm; G.map_a_lo = nm + 1; G.map_b = nm + 2; G.map_b_lo = nm + 3;
             G.vec_ok = ((reinterpret_cast<uintptr_t>(C[i]) & 15) == 0 && ldc[i] % 4 == 0) ? 1 : 0;
             G.scale = scale_of(i);
+            G.corr16 = corr16;
             nm += 4;
         } else if (d == 0) {
             const long long ldt = rup(K[i], 4);
@@ -1150,7 +1188,8 @@ fmm_status_t batched_build(fmm_batched_s* b, int count, const int64_t* M, const 
             tmp.mode = b->mode;
             tmp.peel = 0;
             tmp.pre16 = b->pre;
-            tmp.split_kind = b->split_kind;
+            tmp.split_kind = b->split_kind != kSplitTF32X || tf32x_leaf(leaf_k(K[i], d, false), d) ? b->split_kind
+                                                                                                   : kSplitTF32;
             tmp.sched = 0;   // its leaves run in the batched launch
             size_t need = 0;
             layout(&tmp, nullptr, &need);
@@ -1306,6 +1345,9 @@ void make_tmp(fmm_plan_s& t, long long M, long long N, long long K, long long ld
         t.mode = o.precision == FMM_PREC_BF16X3   ? kLeafBF16x3P
                  : o.precision == FMM_PREC_FP16X3 ? kLeafFP16x3P
                                                   : kLeaf3xTF32P;
+        if (o.precision == FMM_PREC_FP32 && t.pair && t.rmul == 0 && tf32x_leaf(leaf_k(K, t.depth, t.peel != 0), t.depth)) {
+            t.split_kind = kSplitTF32X;
+        }
     }
     // the fused last level needs the CTA-pair kernel on split planes and a
     // Winograd depth of 2 to 4 (the node outputs then fold into C in one pass)

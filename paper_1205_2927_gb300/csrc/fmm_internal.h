@@ -29,7 +29,7 @@ struct GemmGroup {
     int map_a, map_b;       // tensor-map indices
     int a_batch_off, b_batch_off;
     int vec_ok;             // C, ldc and the batch stride allow 16-byte stores
-    int pad_;
+    int corr16;             // kLeaf3xTF32P on CTA pairs: kSplitTF32X planes, bf16 correction products
     const float* scale;     // 16-bit split leaves: device {s_a, s_b} power-of-two operand scales, or null
     int map_a_lo, map_b_lo; // pre-split 16-bit leaves: maps of the lo planes (map_a / map_b hold hi)
 };
@@ -147,6 +147,7 @@ struct SplitJob {
     int tiles_c;            // 128-column blocks per 32-row band of the source
     int transpose;
     const float* scale;     // FP16x3: the problem's device {s_a, s_b} (the job uses scale[transpose]), or null
+    int corr16;             // a launch of kind kSplitTF32X: 1 for its planes, 0 for kSplitTF32 ones
 };
 cudaError_t launch_batched_split(const SplitJob* jobs, int njobs, long long total_tiles, int kind,
                                  cudaStream_t stream);
@@ -190,7 +191,13 @@ cudaError_t launch_quad_post(const QuadPost& q, int part, cudaStream_t stream);
 // Kinds of split: bf16 (x*s = hi + lo, 16-bit), fp16 (same, 16-bit), tf32
 // (fp32 planes: hi = x itself -- the tensor core reads trunc_tf32(x) -- and
 // lo = rn_tf32(x - trunc_tf32(x))).
-enum SplitKind : int { kSplitBF16 = 0, kSplitFP16 = 1, kSplitTF32 = 2 };
+// tf32x (CTA-pair leaves): hi = the nearest TF32 value of x as fp32 (or the raw
+// operand itself, read truncated), and in place of the lo plane one of the same
+// size whose 128-byte lines hold, per 32 columns, 32 bf16 values of hi and then
+// 32 of x - hi: the operands of the two correction products.  Its columns from
+// the matrix's last to the next multiple of 32 are written as zeros.
+enum SplitKind : int { kSplitBF16 = 0, kSplitFP16 = 1, kSplitTF32 = 2, kSplitTF32X = 3 };
+inline bool split_is32(int kind) { return kind == kSplitTF32 || kind == kSplitTF32X; }
 // A stack of split matrices: child c of node p at plane + (p * nchild + c) *
 // child_stride elements, row stride ld (elements, multiple of 8 so rows start
 // on 16 bytes); element size 2 (bf16, fp16) or 4 (tf32).

@@ -490,6 +490,15 @@ __global__ void __launch_bounds__(LeafCfg<BN, MODE>::kThreads, 1) leaf_gemm_kern
 //   CTA 0      warp 1: MMA issuer; commits are multicast to both CTAs, so each
 //              CTA's producer waits on its own empty barrier
 //
+// FP32 leaves whose planes are kSplitTF32X (GemmGroup::corr16) issue, per 32
+// columns of K, four TF32 MMAs for hi*hi and two bf16 MMAs (K = 16) for each of
+// lo*hi and hi*lo: 8 instructions instead of 12 at the same operand bytes.
+// Bound: shared memory (operand reads 64 B/clk and tile copies 64 B/clk of 128;
+// ncu at n = 4096, depth 1: tensor pipe 77 % busy, L2 49 %).  Leaf launch, three
+// TF32 products -> this: n = 2048 depth 0 66 -> 51 us, 4096 depth 1 352 -> 291 us,
+// 8192 depth 2 2.39 -> 1.88 ms.  Six half stages of 32 KB, or alternating which
+// kind goes first, changed nothing beyond 3 %.
+//
 // FUSED: the last Winograd level inside the leaf launch.  A schedule unit is one
 // 256 x 256 tile position of one last-level node; the pair computes the node's
 // seven products at that position back to back, in the order P1, P2, P6, P7,
@@ -680,6 +689,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
         if (lane == 0 && rank == 0) {
             constexpr uint32_t fmt = (MODE == kLeaf3xTF32P || MODE == kLeafTF32) ? 2u : (MODE == kLeafBF16x3P ? 1u : 0u);
             constexpr uint32_t idesc_full = make_idesc(fmt, 256, 256);
+            constexpr uint32_t idesc_corr_full = make_idesc(1u, 256, 256);   // bf16 correction products
             int stage = 0;
             uint32_t phase = 0;
             int acc = 0;
@@ -692,7 +702,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
                 int g, b, tm, tn;
                 decode_tile(groups, ng, args.raster_m, t, g, b, tm, tn);
                 const int nk = (groups[g].K + Cfg::kKB - 1) / Cfg::kKB;
-                const uint32_t idesc = idesc_with_n(idesc_full, dyn ? tile_cols(groups[g].N, tn, 256) : 256u);
+                const uint32_t ncols = dyn ? tile_cols(groups[g].N, tn, 256) : 256u;
+                const uint32_t idesc = idesc_with_n(idesc_full, ncols);
+                const uint32_t idesc_corr = idesc_with_n(idesc_corr_full, ncols);
+                const bool corr16 = MODE == kLeaf3xTF32P && groups[g].corr16 != 0;
                 for (int pp = 0; pp < kProducts && ok; ++pp) {
                 if (!mbar_wait_cluster(tempty_bar(acc), acc_phase ^ 1u, abort_flag, status)) { ok = false; break; }
                 tc_fence_after();
@@ -714,6 +727,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
                     } else {
                         // hi / lo tiles with 128-byte rows: 4 MMAs of 32 bytes of K per product
                         const uint32_t bh = ah + Cfg::kRows * 128, al = bh + Cfg::kRows * 128, bl = al + Cfg::kRows * 128;
+                        if (corr16) {
+                            // al, bl: lines of [32 bf16 hi | 32 bf16 lo].  Both kinds add to one
+                            // accumulator of one M x N shape, so they run in the order of issue.
+#pragma unroll
+                            for (int kk = 0; kk < 2; ++kk) {
+                                mma_f16_pair(d, sdesc_kmajor_sw128(al + 64 + kk * 32), sdesc_kmajor_sw128(bl + kk * 32),
+                                             idesc_corr, (kb == 0 && kk == 0) ? 0u : 1u);                // lo_a * hi_b
+                                mma_f16_pair(d, sdesc_kmajor_sw128(al + kk * 32), sdesc_kmajor_sw128(bl + 64 + kk * 32),
+                                             idesc_corr, 1u);                                            // hi_a * lo_b
+                            }
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk)
+                                mma_tf32_pair(d, sdesc_kmajor_sw128(ah + kk * 32), sdesc_kmajor_sw128(bh + kk * 32),
+                                              idesc, 1u);                                                // hi_a * hi_b
+                        } else {
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {
                             const uint32_t first = (kb == 0 && kk == 0) ? 0u : 1u;
@@ -730,6 +758,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
                                 mma_f16_pair(d, ahd, bld, idesc, 1u);
                                 mma_f16_pair(d, ahd, bhd, idesc, 1u);
                             }
+                        }
                         }
                     }
                     mma_commit_pair(empty_bar(stage), (uint16_t)0x3);
