@@ -2,8 +2,9 @@
 //
 // Three row-times-vector passes, each one block per matrix row with coalesced
 // reads along the row: y = B x (K entries), z = A y (M), w = C x (M), r = w - z.
-// Accumulation in fp32, or in fp64 for the optional refinement (O(mn + mk + kn)
-// fp64 operations: at n = 16384 the fp64 pipe, not HBM, sets its time).  One
+// Accumulation in fp32 (rowdot_kernel), or in fp64 for the optional refinement
+// (rowdot64_kernel: O(mn + mk + kn) fp64 operations; the fp64 pipe, not HBM, sets
+// its time).  One
 // pass over A, B and C: bandwidth-bound in fp32.
 #include "../../include/fmm.h"
 #include "fmm_internal.h"
@@ -69,6 +70,131 @@ __global__ void __launch_bounds__(256) rowdot_kernel(const float* __restrict__ X
     }
 }
 
+// float -> double without the FP64 pipe's conversion instruction: a normal
+// value's bits are moved and its exponent rebiased by integer operations.
+__device__ __forceinline__ bool is_normal(float x) {
+    return (__float_as_uint(x) << 1) - 0x01000000u < 0xFE000000u;
+}
+__device__ __forceinline__ double widen_normal(float x) {
+    const uint32_t u = __float_as_uint(x);
+    return __hiloint2double((int)((((u & 0x7FFFFFFFu) >> 3) + 0x38000000u) | (u & 0x80000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double widen_any(float x) {   // zeros, subnormals, infinities, NaN too
+    double d;
+    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(x));
+    return d;
+}
+template <int N>
+__device__ __forceinline__ void widen(const float (&x)[N], double (&d)[N]) {
+    bool normal = true;
+#pragma unroll
+    for (int i = 0; i < N; ++i) normal = normal && is_normal(x[i]);
+    if (normal) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) d[i] = widen_normal(x[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) d[i] = widen_any(x[i]);
+    }
+}
+
+// rowdot_kernel in fp64: R consecutive rows per block, each with the sums and
+// the order that kernel gives it, so v is read (and a float v widened) once for
+// R rows.  Bound: the FP64 pipe (ncu: 91 % busy), which with one
+// conversion per element of X and of v beside the FMA took 1.72 ms for the three
+// passes at 12000 x 9001 x 10500, and with the FMA alone 0.74 ms.  R = 4 on
+// 16-byte rows (four sums a row), 8 on others (one sum a row; two rows took
+// 1.6 times as long as four); below 304 blocks of that, one row per block.
+template <typename Vec, int R, bool VEC4>
+__global__ void __launch_bounds__(256, 3) rowdot64_kernel(const float* __restrict__ X, long long ld,
+                                                                     long long rows, long long cols,
+                                                                     const Vec* __restrict__ v,
+                                                                     double* __restrict__ out,
+                                                                     const double* __restrict__ sub) {
+    __shared__ double warp_sum[8][R];
+    const long long row0 = (long long)blockIdx.x * R;
+    const int t = threadIdx.x, nr = rows - row0 < R ? (int)(rows - row0) : R;
+    const float* xr[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) xr[r] = X + (row0 + (r < nr ? r : 0)) * ld;   // rows past the end read the first one
+    double a[R][VEC4 ? 4 : 1] = {};
+    long long c0 = 0;
+    if constexpr (VEC4) {
+        const long long groups = cols >> 2;
+#pragma unroll 1
+        for (long long g = t; g < groups; g += 256) {
+            float4 q[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) q[r] = __ldg(reinterpret_cast<const float4*>(xr[r]) + g);
+            double w[4];
+            if constexpr (std::is_same<Vec, float>::value) {
+                const float4 f = __ldg(reinterpret_cast<const float4*>(v) + g);
+                const float ff[4] = {f.x, f.y, f.z, f.w};
+                widen(ff, w);
+            } else {
+                const double2 d0 = __ldg(reinterpret_cast<const double2*>(v) + 2 * g);
+                const double2 d1 = __ldg(reinterpret_cast<const double2*>(v) + 2 * g + 1);
+                w[0] = d0.x; w[1] = d0.y; w[2] = d1.x; w[3] = d1.y;
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float qq[4] = {q[r].x, q[r].y, q[r].z, q[r].w};
+                double d[4];
+                widen(qq, d);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) a[r][i] += d[i] * w[i];
+            }
+        }
+        c0 = groups << 2;
+    }
+#pragma unroll 2
+    for (long long c = c0 + t; c < cols; c += 256) {
+        float q[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) q[r] = __ldg(xr[r] + c);
+        double d[R], w[1];
+        if constexpr (std::is_same<Vec, float>::value) {
+            const float f[1] = {__ldg(v + c)};
+            widen(f, w);
+        } else {
+            w[0] = __ldg(v + c);
+        }
+        widen(q, d);
+#pragma unroll
+        for (int r = 0; r < R; ++r) a[r][0] += d[r] * w[0];
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        double acc = a[r][0];
+        if constexpr (VEC4) acc = (a[r][0] + a[r][1]) + (a[r][2] + a[r][3]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if ((t & 31) == 0) warp_sum[t >> 5][r] = acc;
+    }
+    __syncthreads();
+    if (t < nr) {
+        double s = warp_sum[0][t];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) s += warp_sum[w][t];
+        out[row0 + t] = sub ? s - sub[row0 + t] : s;
+    }
+}
+
+template <typename Vec>
+void rowdot64(const float* X, long long ld, long long rows, long long cols, const Vec* v, double* out,
+              const double* sub, int vec4, cudaStream_t s) {
+    const int R = vec4 ? 4 : 8;
+    const bool wide = rows >= 304LL * R;
+    const unsigned grid = (unsigned)(wide ? (rows + R - 1) / R : rows);
+    if (vec4) {
+        if (wide) rowdot64_kernel<Vec, 4, true><<<grid, 256, 0, s>>>(X, ld, rows, cols, v, out, sub);
+        else rowdot64_kernel<Vec, 1, true><<<grid, 256, 0, s>>>(X, ld, rows, cols, v, out, sub);
+    } else {
+        if (wide) rowdot64_kernel<Vec, 8, false><<<grid, 256, 0, s>>>(X, ld, rows, cols, v, out, sub);
+        else rowdot64_kernel<Vec, 1, false><<<grid, 256, 0, s>>>(X, ld, rows, cols, v, out, sub);
+    }
+}
+
 inline int aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 ? 1 : 0; }
 
 // y = B x ; z = A y ; r = C x - z.  y is kept in the accumulation type: an
@@ -80,13 +206,17 @@ cudaError_t residual_impl(long long M, long long N, long long K, const float* A,
                           double* z, cudaStream_t s) {
     Acc* y = reinterpret_cast<Acc*>(y_ws);   // K entries (the workspace holds K doubles)
     const int vx = aligned16(x), vy = aligned16(y);
-    if (K > 0)
-        rowdot_kernel<Acc, float, Acc><<<(unsigned)K, 256, 0, s>>>(B, ldb, K, N, x, y, nullptr,
-                                                                   vx & aligned16(B) & (ldb % 4 == 0));
-    rowdot_kernel<Acc, Acc, double><<<(unsigned)M, 256, 0, s>>>(A, lda, M, K, y, z, nullptr,
-                                                                vy & aligned16(A) & (lda % 4 == 0));
-    rowdot_kernel<Acc, float, double><<<(unsigned)M, 256, 0, s>>>(C, ldc, M, N, x, r, z,
-                                                                  vx & aligned16(C) & (ldc % 4 == 0));
+    const int bv = vx & aligned16(B) & (ldb % 4 == 0), av = vy & aligned16(A) & (lda % 4 == 0),
+              cv = vx & aligned16(C) & (ldc % 4 == 0);
+    if constexpr (std::is_same<Acc, double>::value) {
+        if (K > 0) rowdot64<float>(B, ldb, K, N, x, y, nullptr, bv, s);
+        rowdot64<double>(A, lda, M, K, y, z, nullptr, av, s);
+        rowdot64<float>(C, ldc, M, N, x, r, z, cv, s);
+    } else {
+        if (K > 0) rowdot_kernel<Acc, float, Acc><<<(unsigned)K, 256, 0, s>>>(B, ldb, K, N, x, y, nullptr, bv);
+        rowdot_kernel<Acc, Acc, double><<<(unsigned)M, 256, 0, s>>>(A, lda, M, K, y, z, nullptr, av);
+        rowdot_kernel<Acc, float, double><<<(unsigned)M, 256, 0, s>>>(C, ldc, M, N, x, r, z, cv);
+    }
     return cudaGetLastError();
 }
 
