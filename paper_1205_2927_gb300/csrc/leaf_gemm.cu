@@ -28,6 +28,11 @@
 
 namespace fmm {
 
+// Output staging of the epilogue warps: 32 rows x 32 columns each, rows 36 floats
+// apart (16-byte reads and writes by rows are free of bank conflicts).
+constexpr int kOutPitch = 36;
+constexpr int kOutBytes = 4 * 32 * kOutPitch * 4;
+
 template <int BN, int MODE>
 struct LeafCfg {
     static constexpr bool kPre32 = MODE == kLeaf3xTF32P;                         // fp32 raw / lo planes via TMA
@@ -47,7 +52,7 @@ struct LeafCfg {
     static constexpr int kTmemCols = 2 * BN;
     static constexpr int kThreads = kSplit ? 384 : 256;
     static constexpr int kBarBytes = 256;
-    static constexpr size_t kSmem = 1024 + (size_t)kStages * (kStageBytes + kLoBytes) + kBarBytes;
+    static constexpr size_t kSmem = 1024 + (size_t)kStages * (kStageBytes + kLoBytes) + kBarBytes + kOutBytes;
     static_assert((3 * kStages + 4) * 8 + 16 <= kBarBytes, "barrier area");
     static_assert(kSmem <= 227 * 1024, "shared memory");
     static_assert(kTmemCols == 256 || kTmemCols == 512, "TMEM columns");
@@ -126,6 +131,59 @@ __device__ __forceinline__ long long seq_read(const unsigned long long* slot, un
             }
         }
     }
+}
+
+// One 32 x 32 chunk of an output tile by one warp: lane r brings row r's 32
+// values; the chunk turns through the warp's staging rows so that every store
+// (and load of C, for beta) covers whole lines: 4 rows x 128 bytes at a time where
+// C allows 16-byte accesses, else one row of 32 floats.  Lanes storing their own
+// rows put 32 separate pieces into each instruction: on rows off the 16-byte
+// grid, 4-byte pieces, a 1900 x 3101 x 1503 leaf launch with beta took 210 us,
+// against 92 us this way (512 uneven products, 16-byte pieces: 5.0 -> 4.7 ms).
+// Stores are evict-first: a launch's products are read only after it, and must
+// not push operand lines out of L2.
+__device__ __forceinline__ void store_chunk(float* buf, const float (&v)[32], float* C, long long ldc, int rows,
+                                            int cols, float beta, bool vec, int lane) {
+    float4* mine = reinterpret_cast<float4*>(buf + lane * kOutPitch);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) mine[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+    __syncwarp();
+    if (vec && cols >= 32) {
+        const int r0 = lane >> 3, c = (lane & 7) * 4;
+        float* p = C + r0 * ldc + c;
+        float4 o[8];
+        if (beta != 0.0f) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (4 * i + r0 < rows) o[i] = *reinterpret_cast<const float4*>(p + 4 * i * ldc);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (4 * i + r0 >= rows) break;
+            float4 x = *reinterpret_cast<const float4*>(buf + (4 * i + r0) * kOutPitch + c);
+            if (beta != 0.0f) { x.x += beta * o[i].x; x.y += beta * o[i].y; x.z += beta * o[i].z; x.w += beta * o[i].w; }
+            __stcs(reinterpret_cast<float4*>(p + 4 * i * ldc), x);
+        }
+    } else if (lane < cols) {
+        float* p = C + lane;
+#pragma unroll 1
+        for (int r = 0; r < rows; r += 8) {
+            float o[8];
+            if (beta != 0.0f) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (r + i < rows) o[i] = p[(r + i) * ldc];
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (r + i >= rows) break;
+                float x = buf[(r + i) * kOutPitch + lane];
+                if (beta != 0.0f) x += beta * o[i];
+                __stcs(p + (r + i) * ldc, x);
+            }
+        }
+    }
+    __syncwarp();   // the staging rows are read before the next chunk's are written
 }
 
 template <int BN, int MODE>
@@ -332,11 +390,11 @@ __global__ void __launch_bounds__(LeafCfg<BN, MODE>::kThreads, 1) leaf_gemm_kern
             bool ok = mbar_wait(tfull_bar(acc), acc_phase, abort_flag, status);
             if (!__all_sync(0xffffffffu, ok)) break;
             tc_fence_after();
-            const int row = tm * kBM + q * 32 + lane;
-            const bool row_ok = row < G.M;
-            float* crow = G.C + (long long)b * G.c_batch_stride + (long long)(row_ok ? row : 0) * G.ldc;
+            const int row0 = tm * kBM + q * 32;
+            const int rows = min(32, G.M - row0);   // <= 0: this warp's rows are padding
+            float* crow = G.C + (long long)b * G.c_batch_stride + (long long)row0 * G.ldc;
+            float* buf = reinterpret_cast<float*>(bar_ptr + Cfg::kBarBytes) + q * 32 * kOutPitch;
             float alpha = G.alpha;
-            const float beta = G.beta;
             if (Cfg::k16 && G.scale) alpha = alpha / (G.scale[0] * G.scale[1]);  // undo the operand scaling
 #pragma unroll 1
             for (int c = 0; c < BN / 32; ++c) {
@@ -344,35 +402,11 @@ __global__ void __launch_bounds__(LeafCfg<BN, MODE>::kThreads, 1) leaf_gemm_kern
                 tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + c * 32), r);
                 tmem_ld_wait();
                 const int col0 = tn * BN + c * 32;
-                if (row_ok && col0 < G.N) {
-                    float* cp = crow + col0;
-                    if (G.vec_ok && col0 + 32 <= G.N) {
+                if (rows > 0 && col0 < G.N) {
+                    float v[32];
 #pragma unroll
-                        for (int j = 0; j < 32; j += 4) {
-                            float4 v;
-                            v.x = alpha * __uint_as_float(r[j + 0]);
-                            v.y = alpha * __uint_as_float(r[j + 1]);
-                            v.z = alpha * __uint_as_float(r[j + 2]);
-                            v.w = alpha * __uint_as_float(r[j + 3]);
-                            if (beta != 0.0f) {
-                                const float4 o = *reinterpret_cast<const float4*>(cp + j);
-                                v.x += beta * o.x; v.y += beta * o.y; v.z += beta * o.z; v.w += beta * o.w;
-                            }
-                            // evict-first: the products are read only after the
-                            // whole launch, and must not push operand lines out of L2
-                            __stcs(reinterpret_cast<float4*>(cp + j), v);
-                        }
-                    } else {
-                        const int lim = min(32, G.N - col0);
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            if (j < lim) {
-                                float v = alpha * __uint_as_float(r[j]);
-                                if (beta != 0.0f) v += beta * cp[j];
-                                cp[j] = v;
-                            }
-                        }
-                    }
+                    for (int j = 0; j < 32; ++j) v[j] = alpha * __uint_as_float(r[j]);
+                    store_chunk(buf, v, crow + col0, G.ldc, rows, G.N - col0, G.beta, G.vec_ok != 0, lane);
                 }
             }
             tc_fence_before();
@@ -535,24 +569,7 @@ __device__ __forceinline__ float4 ld_keep(const float4* a, uint64_t pol) {
     return v;
 }
 
-// One 32-column chunk of a node-output quadrant (rows and columns of the leaf
-// tile; `o` already points at the quadrant's row) from 32 values in v.
-__device__ __forceinline__ void store_quadrant_chunk(float* o, const float (&v)[32], bool row_ok, int col0, int ncols,
-                                                     int vec_ok) {
-    if (!row_ok || col0 >= ncols) return;
-    if (vec_ok && col0 + 32 <= ncols) {
-#pragma unroll
-        for (int j = 0; j < 32; j += 4)
-            __stcs(reinterpret_cast<float4*>(o + j), make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]));
-    } else {
-        const int lim = min(32, ncols - col0);
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-            if (j < lim) o[j] = v[j];
-    }
-}
-
-template <int MODE>
+template <int MODE, bool FUSED>
 struct PairCfg {
     static constexpr bool kPlain = MODE == kLeafTF32;          // fp32 A | B tiles, one product
     static constexpr int kRows = 128;                          // rows per CTA of A and of B^T
@@ -564,7 +581,7 @@ struct PairCfg {
     static constexpr int kTmemCols = 512;                      // 2 x 256-column accumulators
     static constexpr int kBarBytes = 256;
     static constexpr int kThreads = 256;
-    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kBarBytes;
+    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kBarBytes + kOutBytes;
     static_assert((2 * kStages + 4) * 8 + 16 <= kBarBytes, "barrier area");
     static_assert(kSmem <= 227 * 1024, "shared memory");
 };
@@ -572,7 +589,7 @@ struct PairCfg {
 template <int MODE, bool FUSED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
     leaf_gemm_pair_kernel(const __grid_constant__ GemmArgs args) {
-    using Cfg = PairCfg<MODE>;
+    using Cfg = PairCfg<MODE, FUSED>;
     constexpr int kProducts = FUSED ? 7 : 1;   // products per schedule unit
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -796,57 +813,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
             int g, b, tm, tn;
             decode_tile(groups, ng, args.raster_m, t, g, b, tm, tn);
             const GemmGroup& G = groups[g];
-            const int row = tm * 256 + (int)rank * Cfg::kRows + q * 32 + lane;
-            const bool row_ok = row < G.M;
+            const int row0 = tm * 256 + (int)rank * Cfg::kRows + q * 32;
+            const int rows = min(32, G.M - row0);   // <= 0: this warp's rows are padding
+            float* buf = reinterpret_cast<float*>(bar_ptr + Cfg::kBarBytes) + q * 32 * kOutPitch;
             float alpha = G.alpha;
-            const float beta = G.beta;
             if (MODE == kLeafFP16x3P && G.scale) alpha = alpha / (G.scale[0] * G.scale[1]);
             for (int pp = 0; pp < kProducts; ++pp) {
             bool ok = mbar_wait(tfull_bar(acc), acc_phase, abort_flag, status);
             if (!__all_sync(0xffffffffu, ok)) { stop = true; break; }
             tc_fence_after();
             if constexpr (!FUSED) {
-            float* crow = G.C + (long long)b * G.c_batch_stride + (long long)(row_ok ? row : 0) * G.ldc;
+            float* crow = G.C + (long long)b * G.c_batch_stride + (long long)row0 * G.ldc;
 #pragma unroll 1
             for (int c = 0; c < 256 / 32; ++c) {
                 uint32_t r[32];
                 tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * 256 + c * 32), r);
                 tmem_ld_wait();
                 const int col0 = tn * 256 + c * 32;
-                if (row_ok && col0 < G.N) {
-                    float* cp = crow + col0;
-                    if (G.vec_ok && col0 + 32 <= G.N) {
+                if (rows > 0 && col0 < G.N) {
+                    float v[32];
 #pragma unroll
-                        for (int j = 0; j < 32; j += 4) {
-                            float4 v;
-                            v.x = alpha * __uint_as_float(r[j + 0]);
-                            v.y = alpha * __uint_as_float(r[j + 1]);
-                            v.z = alpha * __uint_as_float(r[j + 2]);
-                            v.w = alpha * __uint_as_float(r[j + 3]);
-                            if (beta != 0.0f) {
-                                const float4 o = *reinterpret_cast<const float4*>(cp + j);
-                                v.x += beta * o.x; v.y += beta * o.y; v.z += beta * o.z; v.w += beta * o.w;
-                            }
-                            // evict-first: the products are read only after the
-                            // whole launch, and must not push operand lines out of L2
-                            __stcs(reinterpret_cast<float4*>(cp + j), v);
-                        }
-                    } else {
-                        const int lim = min(32, G.N - col0);
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            if (j < lim) {
-                                float v = alpha * __uint_as_float(r[j]);
-                                if (beta != 0.0f) v += beta * cp[j];
-                                cp[j] = v;
-                            }
-                        }
-                    }
+                    for (int j = 0; j < 32; ++j) v[j] = alpha * __uint_as_float(r[j]);
+                    store_chunk(buf, v, crow + col0, G.ldc, rows, G.N - col0, G.beta, G.vec_ok != 0, lane);
                 }
             }
             } else {
             // node output: quadrant (qi, qj) at rows qi * M + row, columns qj * N + col
-            float* node = G.C + (long long)b * G.c_batch_stride + (long long)(row_ok ? row : 0) * G.ldc;
+            float* node = G.C + (long long)b * G.c_batch_stride + (long long)row0 * G.ldc;
             const long long qrow = (long long)G.M * G.ldc;
 #pragma unroll 1
             for (int c = 0; c < 256 / 32; ++c) {
@@ -885,7 +878,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
                         o[4 * jj + 2] = y[jj].z + v[4 * jj + 2];
                         o[4 * jj + 3] = y[jj].w + v[4 * jj + 3];
                     }
-                    store_quadrant_chunk(node + qrow + G.N + col0, o, row_ok, col0, G.N, G.vec_ok);
+                    if (rows > 0 && col0 < G.N)
+                        store_chunk(buf, o, node + qrow + G.N + col0, G.ldc, rows, G.N - col0, 0.0f, G.vec_ok != 0, lane);
                 } else {                                            // P2 -> C11, P3 -> C12 (from X); P4 -> C21 (from Y)
                     const float4* src = pp == 6 ? ys : xs;
                     float4 x[8];
@@ -909,7 +903,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
                         }
                     }
                     float* dst = pp == 1 ? node : pp == 5 ? node + G.N : node + qrow;
-                    store_quadrant_chunk(dst + col0, o, row_ok, col0, G.N, G.vec_ok);
+                    if (rows > 0 && col0 < G.N)
+                        store_chunk(buf, o, dst + col0, G.ldc, rows, G.N - col0, 0.0f, G.vec_ok != 0, lane);
                 }
             }
             }
@@ -937,7 +932,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
 
 template <int MODE, bool FUSED>
 static cudaError_t launch_pair_impl(const GemmArgs& args, int num_sms, cudaStream_t stream) {
-    using Cfg = PairCfg<MODE>;
+    using Cfg = PairCfg<MODE, FUSED>;
     auto kern = leaf_gemm_pair_kernel<MODE, FUSED>;
     static bool attr_done[64] = {};
     int dev = 0;
