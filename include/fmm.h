@@ -352,26 +352,24 @@ fmm_status_t fmm_set_cost_model(const float* params, const float* mean6, const f
  * synchronising free.
  *
  * Computes C <- alpha * A * B + beta * C (row-major device pointers, the same
- * conventions as fmm_gemm) with one Winograd level over 3xTF32 tensor-core
- * leaves.  Its temporaries live in a device array of 22,020,352 bytes compiled
- * into the library (held by every GPU that loads it until the process exits),
- * so M, N and K must each be <= 1024; larger sizes return FMM_ERR_INVALID_ARG
- * with the limit in fmm_last_error().  The call allocates nothing (no
- * cudaMalloc/cudaFree, no host heap, no allocating library routine).  The
- * first call on a device looks up the array's device address (once per device,
- * with that device current); make that first call before any stream capture.
- * Every call clears the status word it uses, so fmm_gemm_static_status reports
- * on the last call.  All calls share the one array, which keeps the last
- * call's contents: calls that overlap on the GPU (different streams, or
- * different threads on the same device) race and must be serialised by the
- * caller. */
+ * conventions as fmm_gemm) in one launch over FP32 (3xTF32) tensor-core tiles
+ * whose CTAs split and turn the operands themselves and share long K ranges, so
+ * it needs no temporaries.  M, N and K must each be <= 1024; larger sizes return
+ * FMM_ERR_INVALID_ARG with the limit in fmm_last_error().  The call allocates
+ * nothing (no cudaMalloc/cudaFree, no host heap, no allocating library
+ * routine).  The first call on a device looks up the device address of the
+ * library's status word (once per device, with that device current); make that
+ * first call before any stream capture.  Every call clears the status word, so
+ * fmm_gemm_static_status reports on the last call; calls that overlap on the GPU
+ * (different streams, or different threads on the same device) share that one
+ * word. */
 fmm_status_t fmm_gemm_static(int64_t M, int64_t N, int64_t K, float alpha, const float* A, int64_t lda,
                              const float* B, int64_t ldb, float beta, float* C, int64_t ldc,
                              fmm_stream_t stream);
 
 /* Device status of the last fmm_gemm_static call on the current device:
- * synchronises `stream` (the stream of that call), reads the status word in
- * the library's fixed array and clears it.  FMM_OK, FMM_ERR_TIMEOUT when one
+ * synchronises `stream` (the stream of that call), reads the library's status
+ * word and clears it.  FMM_OK, FMM_ERR_TIMEOUT when one
  * of the call's bounded device waits ran out (C is then incomplete), or
  * FMM_ERR_CUDA for any other device-side error bit.  Allocates nothing. */
 fmm_status_t fmm_gemm_static_status(fmm_stream_t stream);

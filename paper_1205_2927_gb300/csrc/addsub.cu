@@ -478,12 +478,6 @@ __global__ void __launch_bounds__(128) quad_post_kernel(QuadPost q) {
 // must not push out the operand lines a fused pass reads again.
 //   tf32x:       hi = rn_tf32(x) (trunc_tf32(x) where the leaves read the raw operand), and in the
 //                other plane bf16(hi) and bf16(x - hi), 32 columns of each per 128-byte line
-// Nearest TF32 value (ties away from zero); what would round past the largest
-// finite value, and infinities, keep their truncation.
-__device__ __forceinline__ float tf32x_hi(float x) {
-    const uint32_t u = __float_as_uint(x), r = (u + 0x1000u) & 0xFFFFE000u;
-    return __uint_as_float((r & 0x7F800000u) == 0x7F800000u ? (u & 0xFFFFE000u) : r);
-}
 // Two values to bf16, nearest even, saturating at the largest finite value.
 __device__ __forceinline__ uint32_t bf16x2_sat(float x0, float x1) {
     uint32_t r;
@@ -498,7 +492,7 @@ __device__ __forceinline__ void split_store(void* hi_plane, void* lo_plane, long
     if constexpr (KIND == kSplitTF32X) {
         float4 h;
         if (hi_plane) {
-            h = f4(tf32x_hi(v.x), tf32x_hi(v.y), tf32x_hi(v.z), tf32x_hi(v.w));
+            h = f4(tf32_round_hi(v.x), tf32_round_hi(v.y), tf32_round_hi(v.z), tf32_round_hi(v.w));
             __stcs(reinterpret_cast<float4*>(static_cast<float*>(hi_plane) + o), h);
         } else {
             h = f4(tf32_trunc(v.x), tf32_trunc(v.y), tf32_trunc(v.z), tf32_trunc(v.w));
@@ -789,7 +783,7 @@ __device__ __forceinline__ float child_of1(int i, float Q0, float Q1, float Q2, 
 template <int KIND>
 __device__ __forceinline__ void split_store1(void* hi_plane, void* lo_plane, long long o, float v, float sc) {
     if constexpr (KIND == kSplitTF32X) {
-        const float hv = tf32x_hi(v);
+        const float hv = tf32_round_hi(v);
         const uint32_t p = bf16x2_sat(hv, v - hv);
         unsigned short* hl = static_cast<unsigned short*>(lo_plane) + tf32x_off(o);
         __stcs(static_cast<float*>(hi_plane) + o, hv);

@@ -175,6 +175,8 @@ struct fmm_plan_s {
     int split_kind = 0;
     int pair = 0;        // leaves on CTA pairs (cta_group::2), 256 x 256 tiles
     int tile_req = 256;  // leaf tile the plan was made for (512: CTA pairs where the precision allows)
+    int small_bn = 0;    // depth 0 in one launch of small_gemm.cu: its tile width (0: the leaf path)
+    int small_splits = 1;
     int rmul = 0;        // classical recursion (Table 1) depth; the Winograd depth is then 0
     // the last Winograd level inside the leaf launch (CTA pairs, split planes,
     // depth 2 to 4): the launch writes the level-(d-1) node outputs, not the
@@ -182,7 +184,7 @@ struct fmm_plan_s {
     int fused = 0;
     float* fuse_scratch = nullptr;
     char* tile_sched = nullptr;   // dynamic tile order of the leaf launches (counter + rings)
-    int sched = 1;                // 0: static tile order, no scheduling area (the allocation-free entry)
+    int sched = 1;                // 0: no scheduling area (sub-plans of a batched launch)
     void* a16[2] = {};   // hi, lo planes of the leaf A operands (stack or the whole A)
     void* b16[2] = {};   // hi, lo planes of the leaf B^T operands
     long long ld16 = 0;
@@ -489,6 +491,63 @@ bool dynamic_order(const fmm_plan_s* p, const GemmArgs& args) {
         leaves += args.groups[g].batch;
     }
     return leaves > 1;
+}
+
+// One-launch kernel of small products (small_gemm.cu) against the leaf path, both
+// by time models in microseconds fitted to measurements at K = 256 .. 11644:
+//   small  7 + waves * (2 + steps of 32 columns / splits * c), c the step of a
+//          128 x {32, 64, 128} tile
+//   leaf   launches, operand passes at 6 TB/s, waves * (4 + K * k)
+// (FP32 512^3 10.5 us against 31, 573 x 452 x 2103 25 against 74, 1024^3 21
+// against 37; not taken: 1500^3 45 against 48, 900 x 4000 x 1000 62 against 50).
+// Splitting K shortens the accumulators' chains; it is limited to chains whose
+// results then move by less than 2e-5 (FP32: 1.9e-8 per instruction, three per 8
+// columns).  Returns the tile width, or 0 for the leaf path.
+struct SmallModel { double c[3], k, k_pair, launches; int a_bytes, b_bytes, split_k; };
+int small_choice(long long M, long long N, long long K, long long lda, fmm_precision_t prec, bool pair, int min_splits,
+                 bool against_leaf, int* splits) {
+    static const SmallModel models[3] = {{{0.62, 0.66, 0.80}, 0.0285, 0.0175, 13.0, 8, 12, 2048},     // FP32
+                                         {{0.35, 0.38, 0.48}, 0.0145, 0.0085, 11.0, 0, 8, 6144},      // TF32
+                                         {{0.45, 0.50, 0.90}, 0.0135, 0.0135, 13.0, 8, 8, 4096}};     // 16-bit splits
+    const SmallModel& m = models[prec == FMM_PREC_FP32 ? 0 : prec == FMM_PREC_TF32 ? 1 : 2];
+    const double tiles_m = (double)((M + 127) / 128);
+    double best = 1e300;
+    int best_bn = 0;
+    for (int i = 0; i < 3; ++i) {
+        const int bn = 32 << i;
+        const double tiles = tiles_m * (double)((N + bn - 1) / bn);
+        for (int sp = 1; sp <= 8; sp *= 2) {
+            if (sp < min_splits || (sp > 1 && ((K + 31) / 32 < sp || (sp > min_splits && K * (sp - 1) > (long long)m.split_k * sp))))
+                continue;
+            const double resident = sp == 8 ? 128.0 : sp == 4 ? 144.0 : 152.0;   // CTAs whose clusters fit at once
+            const double steps = std::ceil(std::ceil((double)K / 32.0) / sp);
+            const double c = m.c[i] * (lda % 4 ? 1.2 : 1.0);   // rows off the 16-byte grid load by 4 bytes
+            const double t = 7.0 + std::ceil(tiles * sp / resident) * (2.0 + steps * c);
+            if (t < best) {
+                best = t;
+                best_bn = bn;
+                *splits = sp;
+            }
+        }
+    }
+    if (!against_leaf) return best_bn;
+    const double tm = pair ? 256.0 : 128.0, slots = pair ? 76.0 : 152.0;
+    const double waves = std::ceil(std::ceil((double)M / tm) * std::ceil((double)N / 256.0) / slots);
+    const double leaf = m.launches + ((double)M * K * m.a_bytes + (double)K * N * m.b_bytes) / 6e6 +
+                        waves * (4.0 + (double)K * (pair ? m.k_pair : m.k));
+    return best < 0.85 * leaf ? best_bn : 0;   // the models miss by up to 15 %
+}
+
+SmallArgs small_args(long long M, long long N, long long K, float alpha, const float* A, long long lda, const float* B,
+                     long long ldb, float beta, float* C, long long ldc, unsigned* status) {
+    SmallArgs a;
+    memset(&a, 0, sizeof(a));
+    a.A = A; a.B = B; a.C = C;
+    a.lda = lda; a.ldb = ldb; a.ldc = ldc;
+    a.M = (int)M; a.N = (int)N; a.K = (int)K;
+    a.alpha = alpha; a.beta = beta;
+    a.status = status;
+    return a;
 }
 
 // Leaf launch over `groups` (already filled except tile bookkeeping).
@@ -978,6 +1037,19 @@ fmm_status_t execute(fmm_plan_s* p, float alpha, const float* A, const float* B,
         p->launches += 3;
         p->acct[0] += 4.0 * (double)(p->M * p->K + p->K * p->N);
     }
+    if (p->small_bn) {
+        SmallArgs a = small_args(p->M, p->N, p->K, alpha, A, p->lda, B, p->ldb, beta, C, p->ldc, p->status);
+        if (p->opt.precision == FMM_PREC_FP16X3) a.scale = p->fp16_scale();
+        const int mode = p->opt.precision == FMM_PREC_TF32     ? kSmallTF32
+                         : p->opt.precision == FMM_PREC_BF16X3 ? kSmallBF16x3
+                         : p->opt.precision == FMM_PREC_FP16X3 ? kSmallFP16x3
+                                                               : kSmall3xTF32;
+        mark(p, 1, stream);
+        FMM_CUDA(launch_small_gemm(a, mode, p->small_bn, p->small_splits, stream));
+        p->launches += 1;
+        mark(p, 2, stream);
+        return FMM_OK;
+    }
     return (p->depth == 0) ? run_classical(p, alpha, A, B, beta, C, stream)
                            : run_winograd(p, alpha, A, B, beta, C, stream);
 }
@@ -1287,8 +1359,10 @@ fmm_status_t batched_check(int count, const int64_t* M, const int64_t* N, const 
 namespace {
 
 // ----------------------------------------------------------------------------------------- planner
+// `outer`: recursion levels above the plan's root (1: the child of a host-resident
+// plan, whose leaves are then those of the device-resident plan one level deeper).
 void make_tmp(fmm_plan_s& t, long long M, long long N, long long K, long long lda, long long ldb, long long ldc,
-              const fmm_options_t& o, int depth, int bn) {
+              const fmm_options_t& o, int depth, int bn, int outer = 0) {
     t.M = M; t.N = N; t.K = K; t.lda = lda; t.ldb = ldb; t.ldc = ldc;
     t.opt = o;
     t.host = o.host_operands ? 1 : 0;
@@ -1345,10 +1419,18 @@ void make_tmp(fmm_plan_s& t, long long M, long long N, long long K, long long ld
         t.mode = o.precision == FMM_PREC_BF16X3   ? kLeafBF16x3P
                  : o.precision == FMM_PREC_FP16X3 ? kLeafFP16x3P
                                                   : kLeaf3xTF32P;
-        if (o.precision == FMM_PREC_FP32 && t.pair && t.rmul == 0 && tf32x_leaf(leaf_k(K, t.depth, t.peel != 0), t.depth)) {
+        if (o.precision == FMM_PREC_FP32 && t.pair && t.rmul == 0 && tf32x_leaf(leaf_k(K, t.depth, t.peel != 0), t.depth + outer)) {
             t.split_kind = kSplitTF32X;
         }
     }
+    // depth 0 with the leaf tile left open: small products in one launch where the
+    // models favour it.  Planners that time tiles reach it by their 256 candidate;
+    // a caller who fixes depth 0 for leaves of 1024 and more keeps the leaf path,
+    // whose operand passes fmm_plan_phase_bytes reports
+    t.small_bn = 0;
+    if (!t.host && outer == 0 && t.depth == 0 && t.rmul == 0 && o.leaf_tile == 0 && M > 0 && N > 0 && K > 0 &&
+        (o.planner == FMM_PLANNER_FIXED || bn == 256) && (std::min(M, N) < 1024 || o.depth < 0))
+        t.small_bn = small_choice(M, N, K, lda, o.precision, bn == 512, 1, true, &t.small_splits);
     // the fused last level needs the CTA-pair kernel on split planes and a
     // Winograd depth of 2 to 4 (the node outputs then fold into C in one pass)
     const bool fusable = t.pair && t.pre16 && !t.host && t.rmul == 0 && t.depth >= 2 && t.depth <= 4;
@@ -1427,7 +1509,14 @@ void make_child(const fmm_plan_s* p, fmm_plan_s& c) {
     fmm_options_t o = p->opt;
     o.host_operands = 0;
     o.odd = FMM_ODD_PAD;   // the quadrant buffers are padded to the level granule already
-    make_tmp(c, p->hm, p->hn, p->hk, p->hk, p->hn, p->hn, o, p->depth > 0 ? p->depth - 1 : 0, p->tile_req);
+    make_tmp(c, p->hm, p->hn, p->hk, p->hk, p->hn, p->hn, o, p->depth > 0 ? p->depth - 1 : 0, p->tile_req,
+             p->depth > 0 ? 1 : 0);
+    if (p->depth == 0) {   // the kernel a device-resident plan of the unpadded sizes takes
+        fmm_plan_s d;
+        make_tmp(d, p->M, p->N, p->K, p->K, p->N, p->N, o, 0, p->tile_req);
+        c.small_bn = d.small_bn;
+        c.small_splits = d.small_splits;
+    }
 }
 
 // Host-resident multiply.  The root level runs depth-first over the seven
@@ -1607,7 +1696,10 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
 
 // Score the candidates with the registered network (one inference launch) and
 // return the index of the smallest predicted time (ties: smaller depth, then
-// the larger tile).
+// the larger tile).  The fixed rule's plan is kept unless that is predicted to
+// take a fifth less: predictions miss by several percent (more where tiles
+// quantise), and the fixed rule is within 1 % of the best candidate over 60
+// unseen shapes.
 fmm_status_t choose_mlp(long long M, long long N, long long K, const fmm_options_t& o, const Cand* c, int n,
                         int* best, cudaStream_t stream) {
     int dev = 0;
@@ -1640,6 +1732,9 @@ fmm_status_t choose_mlp(long long M, long long N, long long K, const fmm_options
         if (d < -1e-6f) b = i;
         else if (d <= 1e-6f && (c[i].depth < c[b].depth || (c[i].depth == c[b].depth && c[i].bn > c[b].bn))) b = i;
     }
+    const int fixed = fixed_depth(M, N, K, o.cutoff), tile = o.leaf_tile ? o.leaf_tile : auto_tile(M, N, fixed, o);
+    for (int i = 0; i < n; ++i)   // outputs are log(ms)
+        if (c[i].depth == fixed && c[i].bn == tile && Y[b] > Y[i] - 0.223f) b = i;
     *best = b;
     return FMM_OK;
 }
@@ -1659,6 +1754,7 @@ fmm_status_t autotune_core(long long M, long long N, long long K, const fmm_opti
         fmm_plan_s t;
         fmm_options_t od = o;
         od.host_operands = 0;   // candidates are timed on device operands
+        od.planner = FMM_PLANNER_EXHAUSTIVE;   // each tile as itself (make_tmp)
         make_tmp(t, M, N, K, K, N, N, od, c[i].depth, c[i].bn);
         size_t need = 0;
         layout(&t, nullptr, &need);
@@ -2453,34 +2549,30 @@ fmm_status_t fmm_plan_info(fmm_plan_t p, int* depth, int* leaf_tile, int* precis
 }  // extern "C"
 
 // ------------------------------------------------------------------------------------------
-// Allocation-free entry point.  Its temporaries (child operands of one Winograd
-// level and the seven products) live in a fixed device array compiled into the
-// library, so the call needs no workspace from the caller and makes no device
-// or host allocation.  The array is shared by every call on a device: calls
-// that overlap on the GPU race on it.
+// Allocation-free entry point: one launch of the small-product kernel, which needs
+// no temporaries; only its status word lives in device memory compiled into the
+// library.  Calls that overlap on the GPU share that word.
 namespace {
 constexpr long long kStaticMaxDim = 1024;
-// status block + 7 child operands per side + 7 products, each (1024/2)^2 floats
-constexpr size_t kStaticBytes = 256 + 3 * (size_t)7 * (kStaticMaxDim / 2) * (kStaticMaxDim / 2) * sizeof(float);
-__device__ __align__(256) unsigned char g_static_scratch[kStaticBytes];
-// device address of the array, per device; filled on a device's first call and
+__device__ __align__(256) unsigned g_static_status[64];
+// device address of the word, per device; filled on a device's first call and
 // read under g_mu, so host threads making first calls at once do not race
-void* g_static_scratch_addr[64] = {};
+unsigned* g_static_status_addr[64] = {};
 
-// The array's device address on the current device (looked up once per device,
+// The word's device address on the current device (looked up once per device,
 // with that device current: the host-side name of the array is not a device
 // address).
-fmm_status_t static_scratch(void** out) {
+fmm_status_t static_status(unsigned** out) {
     int dev = 0;
     FMM_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return FMM_ERR_NO_DEVICE;
     std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_static_scratch_addr[dev]) {
+    if (!g_static_status_addr[dev]) {
         void* ptr = nullptr;
-        FMM_CUDA(cudaGetSymbolAddress(&ptr, g_static_scratch));
-        g_static_scratch_addr[dev] = ptr;
+        FMM_CUDA(cudaGetSymbolAddress(&ptr, g_static_status));
+        g_static_status_addr[dev] = static_cast<unsigned*>(ptr);
     }
-    *out = g_static_scratch_addr[dev];
+    *out = g_static_status_addr[dev];
     return FMM_OK;
 }
 }  // namespace
@@ -2492,8 +2584,7 @@ extern "C" fmm_status_t fmm_gemm_static(int64_t M, int64_t N, int64_t K, float a
     if (M < 0 || N < 0 || K < 0) return FMM_ERR_INVALID_ARG;
     if (M > kStaticMaxDim || N > kStaticMaxDim || K > kStaticMaxDim) {
         snprintf(g_last_error, sizeof(g_last_error),
-                 "fmm_gemm_static: M, N, K must each be <= %lld (static scratch of %zu bytes)", kStaticMaxDim,
-                 kStaticBytes);
+                 "fmm_gemm_static: M, N, K must each be <= %lld", kStaticMaxDim);
         return FMM_ERR_INVALID_ARG;
     }
     if (lda < (K > 0 ? K : 1) || ldb < (N > 0 ? N : 1) || ldc < (N > 0 ? N : 1)) return FMM_ERR_INVALID_ARG;
@@ -2502,49 +2593,36 @@ extern "C" fmm_status_t fmm_gemm_static(int64_t M, int64_t N, int64_t K, float a
     DeviceInfo di;
     fmm_status_t s = device_info(&di);
     if (s != FMM_OK) return s;
-    void* scratch = nullptr;
-    if ((s = static_scratch(&scratch)) != FMM_OK) return s;
+    unsigned* status = nullptr;
+    if ((s = static_status(&status)) != FMM_OK) return s;
     if (alpha == 0.0f || K == 0) {
         // no kernel of this call can report into the status word: clear it so
         // that fmm_gemm_static_status describes this call
-        FMM_CUDA(cudaMemsetAsync(scratch, 0, 64 * sizeof(unsigned), stream));
+        FMM_CUDA(cudaMemsetAsync(status, 0, sizeof(unsigned), stream));
         FMM_CUDA(launch_scale(C, ldc, M, N, beta, stream));
         return FMM_OK;
     }
     if (!A || !B) return FMM_ERR_INVALID_ARG;
-    fmm_options_t o;
-    fmm_options_default(&o);
-    o.depth = 1;
-    fmm_plan_s p;
-    make_tmp(p, M, N, K, lda, ldb, ldc, o, 1, 256);
-    // leaves split their fp32 tiles in shared memory: the temporaries are then
-    // the 7 child operands per side and the 7 products, which the array holds
-    p.pre16 = 0;
-    p.mode = kLeaf3xTF32;
-    p.sched = 0;   // static tile order: no scheduling area in the fixed scratch
-    size_t need = 0;
-    layout(&p, nullptr, &need);
-    if (need > kStaticBytes) return FMM_ERR_WORKSPACE;
-    p.ws = static_cast<char*>(scratch);
-    p.ws_bytes = kStaticBytes;
-    p.num_sms = di.num_sms;
-    layout(&p, p.ws, nullptr);
-    // the array keeps the previous call's contents: the status word must start at zero
-    FMM_CUDA(cudaMemsetAsync(p.status, 0, 64 * sizeof(unsigned), stream));
-    return execute(&p, alpha, A, B, beta, C, stream);
+    // K shared by at least two CTAs beyond one step: its accumulator chains are then
+    // no longer than those of one Winograd level's leaves
+    SmallArgs a = small_args(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, status);
+    a.clear_status = 1;
+    int splits = 1;
+    const int bn = small_choice(M, N, K, lda, FMM_PREC_FP32, false, K > 32 ? 2 : 1, false, &splits);
+    FMM_CUDA(launch_small_gemm(a, kSmall3xTF32, bn, splits, stream));
+    return FMM_OK;
 }
 
 extern "C" fmm_status_t fmm_gemm_static_status(fmm_stream_t stream) {
     DeviceInfo di;
     fmm_status_t s = device_info(&di);
     if (s != FMM_OK) return s;
-    void* scratch = nullptr;
-    if ((s = static_scratch(&scratch)) != FMM_OK) return s;
+    unsigned* status = nullptr;
+    if ((s = static_status(&status)) != FMM_OK) return s;
     FMM_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
     unsigned w = 0;
-    // the status word is the first word of the array (the layout's first carve-out)
-    FMM_CUDA(cudaMemcpy(&w, scratch, sizeof(w), cudaMemcpyDeviceToHost));
-    if (w) FMM_CUDA(cudaMemset(scratch, 0, sizeof(unsigned)));
+    FMM_CUDA(cudaMemcpy(&w, status, sizeof(w), cudaMemcpyDeviceToHost));
+    if (w) FMM_CUDA(cudaMemset(status, 0, sizeof(unsigned)));
     if (w & FMM_DEV_TIMEOUT_BIT) return FMM_ERR_TIMEOUT;
     return w ? FMM_ERR_CUDA : FMM_OK;
 }

@@ -72,6 +72,23 @@ size_t leaf_smem_bytes(int mode, int bn);
 // tiles_n must be counted in 256-row / 256-column units, B maps with 128-row
 // boxes).
 cudaError_t launch_leaf_gemm_pair(const GemmArgs& args, int mode, int num_sms, cudaStream_t stream);
+// One-launch GEMM of a small product (small_gemm.cu): C = alpha A B + beta C,
+// row-major fp32, any alignment.  Tiles of 128 x bn (bn 32, 64 or 128); splits (1,
+// 2, 4 or 8): CTAs of a cluster that share a tile's K range.  The launch fills the
+// fields below `status`.
+enum SmallMode : int { kSmall3xTF32 = 0, kSmallTF32 = 1, kSmallBF16x3 = 2, kSmallFP16x3 = 3 };
+struct SmallArgs {
+    const float *A, *B;
+    float* C;
+    long long lda, ldb, ldc;
+    int M, N, K;
+    float alpha, beta;
+    const float* scale;      // FP16x3: device {s_a, s_b}, or null
+    unsigned* status;        // device status word
+    int clear_status;        // 1: the launch starts its status word from zero
+    int splits, k_chunk, tiles_m, tiles_n, a_vec, c_vec;
+};
+cudaError_t launch_small_gemm(SmallArgs a, int mode, int bn, int splits, cudaStream_t stream);
 // One bounded wait on a barrier nothing signals: sets the timeout bit of *status
 // after limit_ns and returns (the failure path of every pipeline wait).
 cudaError_t launch_wait_selftest(unsigned* status, unsigned long long limit_ns, cudaStream_t stream);

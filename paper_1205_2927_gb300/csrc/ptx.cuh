@@ -314,6 +314,13 @@ __device__ __forceinline__ void tmem_ld_wait() {
 // The TF32 value the tensor core reads from an fp32 operand (low 13 bits cleared).
 __device__ __forceinline__ float tf32_trunc(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
 
+// Nearest TF32 value (ties away from zero); what would round past the largest
+// finite value, infinities and NaN keep their truncation.
+__device__ __forceinline__ float tf32_round_hi(float x) {
+    const uint32_t u = __float_as_uint(x), r = (u + 0x1000u) & 0xFFFFE000u;
+    return __uint_as_float((r & 0x7F800000u) == 0x7F800000u ? (u & 0xFFFFE000u) : r);
+}
+
 // Round an fp32 value to the nearest TF32 value (10 explicit mantissa bits),
 // ties to even, by integer arithmetic on the bit pattern.  Finite inputs.
 __device__ __forceinline__ float tf32_round_rne(float x) {
