@@ -542,81 +542,6 @@ __host__ __device__ __forceinline__ long long plane_cols(long long cols) {
     return KIND == kSplitTF32X ? (cols + 31) & ~31LL : cols;
 }
 
-// Same arithmetic as pre_add_kernel (all 7 children), output split into planes.
-template <bool VEC, int SIDE_B, int KIND>
-__global__ void __launch_bounds__(128) pre_add16_kernel(View P, long long h, long long w, Stack16 out,
-                                                        const float* __restrict__ scale) {
-    const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-    if (c >= plane_cols<KIND>(w)) return;
-    const float sc = scale ? scale[SIDE_B] : 1.0f;
-    const long long node = blockIdx.z;
-    if (c >= w) P.valid_rows = 0;   // padding columns of a tf32x plane: zeros
-    const float* base = P.ptr + node * P.node_stride;
-    const float* q1p = base + w;
-    const float* q2p = base + h * P.ld;
-    const float* q3p = q2p + w;
-    View v0 = P, v1 = P, v2 = P, v3 = P;
-    v1.valid_cols = P.valid_cols - w;
-    v2.valid_rows = P.valid_rows - h;
-    v3.valid_rows = P.valid_rows - h;
-    v3.valid_cols = P.valid_cols - w;
-    for (long long r = blockIdx.y; r < h; r += gridDim.y) {
-        const float4 Q0 = load_q<VEC>(v0, base, r, c);
-        const float4 Q1 = load_q<VEC>(v1, q1p, r, c);
-        const float4 Q2 = load_q<VEC>(v2, q2p, r, c);
-        const float4 Q3 = load_q<VEC>(v3, q3p, r, c);
-        float4 X1, X2, X3, X4;
-        if (!SIDE_B) {
-            X1 = add4(Q2, Q3); X2 = sub4(X1, Q0); X3 = sub4(Q0, Q2); X4 = sub4(Q1, X2);
-        } else {
-            X1 = sub4(Q2, Q0); X2 = sub4(Q3, X1); X3 = sub4(Q3, Q2); X4 = sub4(X2, Q1);
-        }
-        const float4 ch[7] = {Q0, Q1, SIDE_B ? Q3 : X4, SIDE_B ? X4 : Q3, X1, X2, X3};
-        const long long o = (node * out.nchild) * out.child_stride + r * out.ld + c;
-#pragma unroll
-        for (int i = 0; i < 7; ++i) split_store<KIND>(out.hi, out.lo, o + i * out.child_stride, ch[i], sc);
-    }
-}
-
-// Root B side into 16-bit planes (transposing), children in product order.
-template <int KIND>
-__global__ void __launch_bounds__(256) pre_add16_b_root_kernel(const float* __restrict__ B, long long ldb, long long K,
-                                                               long long N, long long kh, long long nh, Stack16 out,
-                                                               const float* __restrict__ scale) {
-    __shared__ float tile[7][32][33];
-    const float sc = scale ? scale[1] : 1.0f;
-    const long long k0 = (long long)blockIdx.y * 32, n0 = (long long)blockIdx.x * 32;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int kl = ty + 8 * i;
-        const long long k = k0 + kl, n = n0 + tx;
-        float b11 = 0.f, b12 = 0.f, b21 = 0.f, b22 = 0.f;
-        if (k < kh && n < nh) {
-            const long long kk2 = k + kh, nn2 = n + nh;
-            if (k < K && n < N) b11 = B[k * ldb + n];
-            if (k < K && nn2 < N) b12 = B[k * ldb + nn2];
-            if (kk2 < K && n < N) b21 = B[kk2 * ldb + n];
-            if (kk2 < K && nn2 < N) b22 = B[kk2 * ldb + nn2];
-        }
-        const float t1 = b12 - b11, t2 = b22 - t1, t3 = b22 - b12, t4 = t2 - b21;
-        tile[0][kl][tx] = b11; tile[1][kl][tx] = b21; tile[2][kl][tx] = b22; tile[3][kl][tx] = t4;
-        tile[4][kl][tx] = t1;  tile[5][kl][tx] = t2;  tile[6][kl][tx] = t3;
-    }
-    __syncthreads();
-    // each thread: 4 consecutive k of one n row, for the 7 children
-    const int t = ty * 32 + tx;          // 0..255
-    const int nl = t >> 3, kq = (t & 7) * 4;
-    const long long n = n0 + nl, k = k0 + kq;
-    if (n < nh && k < plane_cols<KIND>(kh)) {
-#pragma unroll
-        for (int c = 0; c < 7; ++c) {
-            const float4 v = make_float4(tile[c][kq][nl], tile[c][kq + 1][nl], tile[c][kq + 2][nl], tile[c][kq + 3][nl]);
-            split_store<KIND>(out.hi, out.lo, c * out.child_stride + n * out.ld + k, v, sc);
-        }
-    }
-}
-
 // Plain split (transpose = 0: rows x cols -> rows x ld planes) or transposed
 // split (transpose = 1: X is rows(K) x cols(N), planes are cols x ld).  Every
 // thread issues all of its loads before its first store.  Plain: one 32 x 128
@@ -698,59 +623,149 @@ __device__ __forceinline__ void children7(const float4 (&Q)[4], float4 (&ch)[7])
     ch[4] = X1; ch[5] = X2; ch[6] = X3;
 }
 
-// Pre-additions of two consecutive levels in one pass: each node operand
-// (4h x 4w, a uniform stack) -> its 49 grandchildren (h x w), written as split
-// planes at stack index (node * 7 + i) * 7 + j.  Identical arithmetic to two
-// pre_add passes; the middle level is never stored.
 // 4 consecutive elements at (row, col) of a view, zero outside its valid window.
-template <bool VEC>
-__device__ __forceinline__ float4 load_sub(const View& v, const float* base, long long row, long long col) {
-    if (VEC && row < v.valid_rows && col + 3 < v.valid_cols)
-        return __ldg(reinterpret_cast<const float4*>(base + row * v.ld + col));
+__device__ __forceinline__ float4 load_sub(const View& v, bool vec, long long row, long long col) {
+    if (vec && row < v.valid_rows && col + 3 < v.valid_cols)
+        return __ldg(reinterpret_cast<const float4*>(v.ptr + row * v.ld + col));
     float t[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) t[j] = (row < v.valid_rows && col + j < v.valid_cols) ? __ldg(base + row * v.ld + col + j) : 0.0f;
+    for (int j = 0; j < 4; ++j) t[j] = (row < v.valid_rows && col + j < v.valid_cols) ? __ldg(v.ptr + row * v.ld + col + j) : 0.0f;
     return f4(t[0], t[1], t[2], t[3]);
 }
 
-template <bool VEC, int SIDE_B, int KIND>
-__global__ void __launch_bounds__(128) pre_add2_kernel(View P, long long h, long long w, Stack16 out,
-                                                       const float* __restrict__ scale) {
-    const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-    if (c >= plane_cols<KIND>(w)) return;
-    if (c >= w) P.valid_rows = 0;   // padding columns of a tf32x plane: zeros
-    const float sc = scale ? scale[SIDE_B] : 1.0f;
-    const long long node = blockIdx.z;
-    const float* base = P.ptr + node * P.node_stride;
-    for (long long r = blockIdx.y; r < h; r += gridDim.y) {
-        // sub-block (a, b) of the node: quadrant (a / 2, b / 2), sub-quadrant (a % 2, b % 2)
-        float4 X[4][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b)
-                X[a][b] = load_sub<VEC>(P, base, a * h + r, b * w + c);
-        // quadrant q of the node, sub-quadrant t: X[(q / 2) * 2 + t / 2][(q % 2) * 2 + t % 2]
-        const long long o0 = (node * 49) * out.child_stride + r * out.ld + c;
-        float4 C[4][7];   // child i's quadrant t (t = sub-quadrant position)
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const float4 Qt[4] = {X[(t >> 1)][(t & 1)], X[(t >> 1)][2 + (t & 1)], X[2 + (t >> 1)][(t & 1)],
-                                  X[2 + (t >> 1)][2 + (t & 1)]};
-            float4 ch[7];
-            children7<SIDE_B>(Qt, ch);
-#pragma unroll
-            for (int i = 0; i < 7; ++i) C[t][i] = ch[i];
-        }
-#pragma unroll
-        for (int i = 0; i < 7; ++i) {
-            const float4 Qi[4] = {C[0][i], C[1][i], C[2][i], C[3][i]};
-            float4 g[7];
-            children7<SIDE_B>(Qi, g);
-#pragma unroll
-            for (int j = 0; j < 7; ++j) split_store<KIND>(out.hi, out.lo, o0 + (i * 7 + j) * out.child_stride, g[j], sc);
+// Child i (product order) of an operand from its four quadrants: the fp32
+// operations of children7 computing only that child.
+template <int SIDE_B>
+__device__ __forceinline__ float4 child_of4(int i, float4 Q0, float4 Q1, float4 Q2, float4 Q3) {
+    if (!SIDE_B) {
+        switch (i) {
+            case 0: return Q0;
+            case 1: return Q1;
+            case 2: return sub4(Q1, sub4(add4(Q2, Q3), Q0));   // S4 = Q1 - S2
+            case 3: return Q3;
+            case 4: return add4(Q2, Q3);                       // S1
+            case 5: return sub4(add4(Q2, Q3), Q0);             // S2 = S1 - Q0
+            default: return sub4(Q0, Q2);                      // S3
         }
     }
+    switch (i) {
+        case 0: return Q0;
+        case 1: return Q1;
+        case 2: return Q3;
+        case 3: return sub4(sub4(Q3, sub4(Q2, Q0)), Q1);       // T4 = T2 - Q1, T2 = Q3 - T1
+        case 4: return sub4(Q2, Q0);                           // T1
+        case 5: return sub4(Q3, sub4(Q2, Q0));                 // T2
+        default: return sub4(Q3, Q2);                          // T3
+    }
+}
+
+// The 7^D children of one position (4 consecutive columns) of an operand's 2^D x 2^D
+// sub-blocks X, split into planes from element offset o0 on, in product order.
+template <int D, int SIDE_B, int KIND>
+__device__ __forceinline__ void emit_children(const float4 (&X)[1 << D][1 << D], const Stack16& out, long long o0,
+                                              float sc) {
+    if constexpr (D == 1) {
+        const float4 Q[4] = {X[0][0], X[0][1], X[1][0], X[1][1]};
+        float4 ch[7];
+        children7<SIDE_B>(Q, ch);
+#pragma unroll
+        for (int i = 0; i < 7; ++i) split_store<KIND>(out.hi, out.lo, o0 + i * out.child_stride, ch[i], sc);
+    } else {
+#pragma unroll 1
+        for (int i = 0; i < 7; ++i) {
+            float4 Q[4], ch[7];   // child i's quadrants, its children
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                Q[q] = child_of4<SIDE_B>(i, X[q >> 1][q & 1], X[q >> 1][2 + (q & 1)], X[2 + (q >> 1)][q & 1],
+                                         X[2 + (q >> 1)][2 + (q & 1)]);
+            children7<SIDE_B>(Q, ch);
+#pragma unroll
+            for (int j = 0; j < 7; ++j)
+                split_store<KIND>(out.hi, out.lo, o0 + (i * 7 + j) * out.child_stride, ch[j], sc);
+        }
+    }
+}
+
+// Pre-additions of a whole depth-1 or depth-2 recursion, both sides in one launch:
+// the caller's A (a view of 2^D h x 2^D w positions, zero outside its valid window)
+// and row-major B (valid K x N, zero outside) -> the 7^D leaf operands of A and of
+// B^T as split planes; the fp32 operations are those of one pass per level, and no
+// level between is stored.
+//   A blocks (the first a_blocks): a thread takes 4 consecutive columns of one leaf
+//     row, 16-byte loads and stores.
+//   B blocks: leaf position (n, k) of B^T sub-block (a, b) is B[b w + k][a h + n].
+//     A block takes 16 (n) x 32 (k) positions, stages the sub-blocks' 32 rows x 64
+//     bytes in shared memory (every load before the first store; 17 floats a row:
+//     the reads are free of bank conflicts) and then, like an A thread, holds 4
+//     consecutive k of one n and stores along k.
+// Bound: HBM.  n = 8192, depth 2, FP32: both sides PRE2_US us (1.91 GB each way of
+// 2.0), against 284 + 334 us for one launch per side whose B pass turned each
+// group of seven outputs through shared memory; n = 1024: 8.3 + 15.4 -> PRE1K_US us.
+constexpr int kRootN = 16, kRootK = 32, kRootPitch = kRootN + 1;
+struct RootB {
+    const float* ptr;
+    long long ld, K, N, h, w;   // valid K x N; leaf h (n) x w (k)
+};
+template <int D, int KIND>
+__global__ void __launch_bounds__(128) pre_root_kernel(View P, long long h, long long w, Stack16 sa, RootB Bm, Stack16 sb,
+                                                       long long a_blocks, long long tiles_n,
+                                                       const float* __restrict__ scale) {
+    constexpr int S = 1 << D;
+    __shared__ float tile[S * S][kRootK][kRootPitch];
+    const int t = threadIdx.x;
+    float4 X[S][S];
+    if ((long long)blockIdx.x < a_blocks) {
+        const bool vec = (reinterpret_cast<uintptr_t>(P.ptr) & 15) == 0 && (P.ld & 3) == 0;
+        const long long w4 = plane_cols<KIND>(w) >> 2, e = (long long)blockIdx.x * 128 + t, r = e / w4;
+        const long long c = (e - r * w4) * 4;
+        if (r >= h) return;
+        if (c >= w) P.valid_rows = 0;   // padding columns of a tf32x plane: zeros
+#pragma unroll
+        for (int a = 0; a < S; ++a)
+#pragma unroll
+            for (int b = 0; b < S; ++b) X[a][b] = load_sub(P, vec, a * h + r, b * w + c);
+        emit_children<D, 0, KIND>(X, sa, r * sa.ld + c, scale ? scale[0] : 1.0f);
+        return;
+    }
+    const long long blk = (long long)blockIdx.x - a_blocks;
+    const long long n0 = blk % tiles_n * kRootN, k0 = blk / tiles_n * kRootK;
+    const bool vec = (reinterpret_cast<uintptr_t>(Bm.ptr) & 15) == 0 && (Bm.ld & 3) == 0;
+    // S * S sub-blocks x 32 rows x 4 groups of 4 floats over 128 threads
+    float4 v[S * S];
+#pragma unroll
+    for (int j = 0; j < S * S; ++j) {
+        const int kr = t >> 2, q = t & 3;              // sub-block j = S a + b
+        const long long k = k0 + kr, n = n0 + 4 * q;   // h is a multiple of 4: n < h covers n + 3
+        const long long row = (j % S) * Bm.w + k, col = (j / S) * Bm.h + n;
+        v[j] = f4(0.f, 0.f, 0.f, 0.f);
+        if (k < Bm.w && n < Bm.h && row < Bm.K && col < Bm.N) {
+            const float* src = Bm.ptr + row * Bm.ld + col;
+            if (vec && col + 3 < Bm.N) {
+                v[j] = __ldg(reinterpret_cast<const float4*>(src));
+            } else {
+                v[j].x = __ldg(src);
+                if (col + 1 < Bm.N) v[j].y = __ldg(src + 1);
+                if (col + 2 < Bm.N) v[j].z = __ldg(src + 2);
+                if (col + 3 < Bm.N) v[j].w = __ldg(src + 3);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < S * S; ++j) {
+        float* d = &tile[j][t >> 2][4 * (t & 3)];
+        d[0] = v[j].x; d[1] = v[j].y; d[2] = v[j].z; d[3] = v[j].w;
+    }
+    __syncthreads();
+    const int nl = t >> 3, kq = (t & 7) * 4;
+    const long long n = n0 + nl, k = k0 + kq;
+    if (n >= Bm.h || k >= plane_cols<KIND>(Bm.w)) return;
+#pragma unroll
+    for (int a = 0; a < S; ++a)
+#pragma unroll
+        for (int b = 0; b < S; ++b)
+            X[a][b] = f4(tile[a * S + b][kq][nl], tile[a * S + b][kq + 1][nl], tile[a * S + b][kq + 2][nl],
+                         tile[a * S + b][kq + 3][nl]);
+    emit_children<D, 1, KIND>(X, sb, n * sb.ld + k, scale ? scale[1] : 1.0f);
 }
 
 // Child i (product order) of an operand from its four quadrants, one element at
@@ -943,72 +958,6 @@ __global__ void __launch_bounds__(256, 2) pre_add3_bt_kernel(const float* __rest
                 split_store1<KIND>(out.hi, out.lo, o0 + (i * 49 + j * 7 + l) * out.child_stride,
                                    child_of1<1>(l, Cj[0], Cj[1], Cj[2], Cj[3]), sc);
         }
-    }
-}
-
-// Root B side of a depth-2 plan in one pass, straight from the caller's
-// row-major B (valid K x N, zero outside) into the 49 leaf operands of B^T,
-// split into planes.  Leaf position (n, k) of B^T sub-block (a, b) is
-// B[b * w + k][a * h + n] (h = N0 / 4, w = K0 / 4).  A 32 (k) x 32 (n) block of
-// positions is loaded coalesced along n; each thread keeps 4 rows (k) packed in
-// the lanes of a float4, so the chain is pre_add2_kernel's, element for
-// element.  Grandchildren leave through a shared tile, transposed, 7 at a time.
-template <int KIND>
-__global__ void __launch_bounds__(256) pre_add2_b_root_kernel(const float* __restrict__ B, long long ldb, long long K,
-                                                              long long N, long long h, long long w, Stack16 out,
-                                                              const float* __restrict__ scale) {
-    __shared__ float tile[7][32][33];
-    const float sc = scale ? scale[1] : 1.0f;
-    const long long k0 = (long long)blockIdx.y * 32, n0 = (long long)blockIdx.x * 32;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const long long n = n0 + tx;
-    float4 X[4][4];   // X[a][b]: sub-block (a, b) of B^T; lane l = row k0 + ty + 8 l
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            float t[4];
-#pragma unroll
-            for (int l = 0; l < 4; ++l) {
-                const long long k = k0 + ty + 8 * l;
-                const long long row = b * w + k, col = a * h + n;
-                t[l] = (k < w && n < h && row < K && col < N) ? __ldg(B + row * ldb + col) : 0.0f;
-            }
-            X[a][b] = f4(t[0], t[1], t[2], t[3]);
-        }
-    const int t = ty * 32 + tx;
-    const int nl = t >> 3, kq = (t & 7) * 4;   // store role: 4 consecutive k of row n0 + nl
-    const long long on = n0 + nl, ok = k0 + kq;
-    const bool store = on < h && ok < plane_cols<KIND>(w);
-#pragma unroll 1
-    for (int i = 0; i < 7; ++i) {
-        float4 Ci[4];   // child i's quadrant t
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float4 Qt[4] = {X[(q >> 1)][(q & 1)], X[(q >> 1)][2 + (q & 1)], X[2 + (q >> 1)][(q & 1)],
-                                  X[2 + (q >> 1)][2 + (q & 1)]};
-            float4 ch[7];
-            children7<1>(Qt, ch);
-            Ci[q] = ch[i];
-        }
-        float4 g[7];
-        children7<1>(Ci, g);
-#pragma unroll
-        for (int j = 0; j < 7; ++j) {
-            tile[j][ty][tx] = g[j].x;
-            tile[j][ty + 8][tx] = g[j].y;
-            tile[j][ty + 16][tx] = g[j].z;
-            tile[j][ty + 24][tx] = g[j].w;
-        }
-        __syncthreads();
-        if (store) {
-#pragma unroll
-            for (int j = 0; j < 7; ++j) {
-                const float4 v = make_float4(tile[j][kq][nl], tile[j][kq + 1][nl], tile[j][kq + 2][nl], tile[j][kq + 3][nl]);
-                split_store<KIND>(out.hi, out.lo, (i * 7 + j) * out.child_stride + on * out.ld + ok, v, sc);
-            }
-        }
-        __syncthreads();
     }
 }
 
@@ -1348,48 +1297,6 @@ cudaError_t launch_quad_post(const QuadPost& q, int part, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_pre_add16(const View& parent, long long nodes, const Stack16& out, int side_b, int kind,
-                             const float* scale, cudaStream_t stream) {
-    const long long h = parent.rows / 2, w = parent.cols / 2;
-    if (h <= 0 || w <= 0 || nodes <= 0) return cudaSuccess;
-    const bool vec = aligned16(parent.ptr) && parent.ld % 4 == 0 && w % 4 == 0 && parent.node_stride % 4 == 0;
-    dim3 grid((unsigned)((w + 4 * 128 - 1) / (4 * 128)), gy(h), (unsigned)nodes);
-#define FMM_PRE16(V, S, K) pre_add16_kernel<V, S, K><<<grid, 128, 0, stream>>>(parent, h, w, out, scale)
-#define FMM_PRE16K(V, S)                                                    \
-    switch (kind) {                                                          \
-        case kSplitBF16: FMM_PRE16(V, S, kSplitBF16); break;                \
-        case kSplitFP16: FMM_PRE16(V, S, kSplitFP16); break;                \
-        case kSplitTF32X: FMM_PRE16(V, S, kSplitTF32X); break;              \
-        default: FMM_PRE16(V, S, kSplitTF32); break;                        \
-    }
-    if (vec) { if (side_b) { FMM_PRE16K(true, 1) } else { FMM_PRE16K(true, 0) } }
-    else     { if (side_b) { FMM_PRE16K(false, 1) } else { FMM_PRE16K(false, 0) } }
-#undef FMM_PRE16K
-#undef FMM_PRE16
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pre_add16_b_root(const float* B, long long ldb, long long K, long long N, long long kh,
-                                    long long nh, const Stack16& out, int kind, const float* scale,
-                                    cudaStream_t stream) {
-    if (kh <= 0 || nh <= 0) return cudaSuccess;
-    dim3 grid((unsigned)((nh + 31) / 32), (unsigned)((kh + 31) / 32));
-    switch (kind) {
-        case kSplitBF16:
-            pre_add16_b_root_kernel<kSplitBF16><<<grid, dim3(32, 8), 0, stream>>>(B, ldb, K, N, kh, nh, out, scale);
-            break;
-        case kSplitFP16:
-            pre_add16_b_root_kernel<kSplitFP16><<<grid, dim3(32, 8), 0, stream>>>(B, ldb, K, N, kh, nh, out, scale);
-            break;
-        case kSplitTF32X:
-            pre_add16_b_root_kernel<kSplitTF32X><<<grid, dim3(32, 8), 0, stream>>>(B, ldb, K, N, kh, nh, out, scale);
-            break;
-        default:
-            pre_add16_b_root_kernel<kSplitTF32><<<grid, dim3(32, 8), 0, stream>>>(B, ldb, K, N, kh, nh, out, scale);
-    }
-    return cudaGetLastError();
-}
-
 cudaError_t launch_split16(const float* X, long long ldx, long long rows, long long cols, const Stack16& out,
                            int transpose, int kind, const float* scale, int which, cudaStream_t stream) {
     if (rows <= 0 || cols <= 0) return cudaSuccess;
@@ -1410,41 +1317,36 @@ cudaError_t launch_split16(const float* X, long long ldx, long long rows, long l
     return cudaGetLastError();
 }
 
-cudaError_t launch_pre_add2(const View& node, long long nodes, const Stack16& out, int side_b, int kind,
-                            const float* scale, cudaStream_t stream) {
-    const long long h = node.rows / 4, w = node.cols / 4;
-    if (h <= 0 || w <= 0 || nodes <= 0) return cudaSuccess;
-    if (w % 4) return cudaErrorInvalidValue;
-    const bool vec = aligned16(node.ptr) && node.ld % 4 == 0 && node.node_stride % 4 == 0;
-    dim3 grid((unsigned)((w + 511) / 512), gy(h), (unsigned)nodes);
-#define FMM_PRE2(V, S, K) pre_add2_kernel<V, S, K><<<grid, 128, 0, stream>>>(node, h, w, out, scale)
-#define FMM_PRE2K(V, S)                                        \
-    switch (kind) {                                             \
-        case kSplitBF16: FMM_PRE2(V, S, kSplitBF16); break;    \
-        case kSplitFP16: FMM_PRE2(V, S, kSplitFP16); break;    \
-        case kSplitTF32X: FMM_PRE2(V, S, kSplitTF32X); break;  \
-        default: FMM_PRE2(V, S, kSplitTF32); break;            \
+template <int D>
+static cudaError_t launch_pre_root_impl(const View& a, const float* B, long long ldb, long long K, long long N,
+                                        long long hb, const Stack16& sa, const Stack16& sb, int kind,
+                                        const float* scale, cudaStream_t stream) {
+    const long long h = a.rows >> D, w = a.cols >> D;
+    if (h <= 0 || w <= 0 || hb <= 0) return cudaSuccess;
+    if (w % 4 || hb % 4) return cudaErrorInvalidValue;
+    const long long wp = kind == kSplitTF32X ? (w + 31) & ~31LL : w;
+    const long long a_blocks = (h * (wp / 4) + 127) / 128, tiles_n = (hb + kRootN - 1) / kRootN;
+    const long long blocks = a_blocks + tiles_n * ((w + kRootK - 1) / kRootK);
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const RootB b{B, ldb, K, N, hb, w};
+#define FMM_ROOT(KIND_) \
+    pre_root_kernel<D, KIND_><<<(unsigned)blocks, 128, 0, stream>>>(a, h, w, sa, b, sb, a_blocks, tiles_n, scale)
+    switch (kind) {
+        case kSplitBF16: FMM_ROOT(kSplitBF16); break;
+        case kSplitFP16: FMM_ROOT(kSplitFP16); break;
+        case kSplitTF32X: FMM_ROOT(kSplitTF32X); break;
+        default: FMM_ROOT(kSplitTF32); break;
     }
-    if (vec) { if (side_b) { FMM_PRE2K(true, 1) } else { FMM_PRE2K(true, 0) } }
-    else     { if (side_b) { FMM_PRE2K(false, 1) } else { FMM_PRE2K(false, 0) } }
-#undef FMM_PRE2K
-#undef FMM_PRE2
+#undef FMM_ROOT
     return cudaGetLastError();
 }
 
-cudaError_t launch_pre_add2_b_root(const float* B, long long ldb, long long K, long long N, long long h, long long w,
-                                   const Stack16& out, int kind, const float* scale, cudaStream_t stream) {
-    if (h <= 0 || w <= 0) return cudaSuccess;
-    if (w % 4) return cudaErrorInvalidValue;
-    dim3 grid((unsigned)((h + 31) / 32), (unsigned)((w + 31) / 32));
-    dim3 block(32, 8);
-    switch (kind) {
-        case kSplitBF16: pre_add2_b_root_kernel<kSplitBF16><<<grid, block, 0, stream>>>(B, ldb, K, N, h, w, out, scale); break;
-        case kSplitFP16: pre_add2_b_root_kernel<kSplitFP16><<<grid, block, 0, stream>>>(B, ldb, K, N, h, w, out, scale); break;
-        case kSplitTF32X: pre_add2_b_root_kernel<kSplitTF32X><<<grid, block, 0, stream>>>(B, ldb, K, N, h, w, out, scale); break;
-        default: pre_add2_b_root_kernel<kSplitTF32><<<grid, block, 0, stream>>>(B, ldb, K, N, h, w, out, scale); break;
-    }
-    return cudaGetLastError();
+cudaError_t launch_pre_root(int depth, const View& a, const float* B, long long ldb, long long K, long long N,
+                            long long hb, const Stack16& sa, const Stack16& sb, int kind, const float* scale,
+                            cudaStream_t stream) {
+    if (depth == 1) return launch_pre_root_impl<1>(a, B, ldb, K, N, hb, sa, sb, kind, scale, stream);
+    if (depth == 2) return launch_pre_root_impl<2>(a, B, ldb, K, N, hb, sa, sb, kind, scale, stream);
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_pre_add3(const View& node, long long nodes, const Stack16& out, int side_b, int kind,

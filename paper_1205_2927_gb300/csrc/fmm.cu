@@ -195,8 +195,8 @@ struct fmm_plan_s {
     // of post-additions run as one pass each; the middle levels are never stored
     bool fuse_pre() const { return pre16 && depth >= 4; }
     bool fuse_post() const { return depth >= 4; }
-    // depth 2: both levels at once from / into the caller's matrices
-    bool fuse_root_pre() const { return pre16 && depth == 2; }
+    // depths 1 and 2: every level at once from, depth 2 into, the caller's matrices
+    bool fuse_root_pre() const { return pre16 && (depth == 1 || depth == 2); }
     bool fuse_root_post() const { return depth == 2; }
     // depth 3: all three levels at once from / into the caller's matrices
     bool fuse_root_pre3() const { return pre16 && depth == 3; }
@@ -336,7 +336,7 @@ void layout(fmm_plan_s* p, char* ws, size_t* needed) {
             L.full = (l < d - 1 || l == 0 || p->pre16) ? 1 : 0;
             const long long per = L.full ? 7 : 4;
             if (p->fuse_pre() && (l == d - 3 || l == d - 2)) continue;   // written by no pass: fused away
-            if (p->fuse_root_pre() && l == 0) continue;   // fused away (both sides read the caller's operands)
+            if (p->fuse_root_pre() && l < d - 1) continue;   // fused away (both sides read the caller's operands)
             if (p->fuse_root_pre3() && l < d - 1) continue;   // fused away (both sides read the caller's operands)
             if (p->pre16 && l == d - 1) {   // the leaves' operands, as split planes
                 p->ld16 = rup(C.k, 128 / (long long)p->es16());   // 128-byte row pitch
@@ -780,34 +780,26 @@ fmm_status_t winograd_pre(fmm_plan_s* p, const float* A, const float* B, cudaStr
         return FMM_OK;
     }
     if (p->fuse_root_pre()) {
-        // both levels at once: root -> the 49 leaf operands; the B side reads the
-        // caller's row-major B and writes the K-major (transposed) leaf planes
-        const Level& Lf = lv[2];
+        // every level at once, both sides in one launch: the caller's A and B -> the
+        // 7^d leaf operands (B's transposed: K-major planes)
+        const Level& Lf = lv[d];
+        const int nleaf = d == 1 ? 7 : 49;
         View va{A, p->lda, 0, p->M0, p->K0, p->Mw, p->Kw};
-        Stack16 sa{p->a16[0], p->a16[1], p->ld16, Lf.m * p->ld16, 49};
-        Stack16 sb{p->b16[0], p->b16[1], p->ld16, Lf.n * p->ld16, 49};
-        FMM_CUDA(launch_pre_add2(va, 1, sa, 0, kind, scale, stream));
-        FMM_CUDA(launch_pre_add2_b_root(B, p->ldb, p->Kw, p->Nw, Lf.n, Lf.k, sb, kind, scale, stream));
-        p->launches += 2;
-        p->acct[0] += root_in + 49.0 * (double)(Lf.m * Lf.k + Lf.n * Lf.k) * pl;
+        Stack16 sa{p->a16[0], p->a16[1], p->ld16, Lf.m * p->ld16, nleaf};
+        Stack16 sb{p->b16[0], p->b16[1], p->ld16, Lf.n * p->ld16, nleaf};
+        FMM_CUDA(launch_pre_root(d, va, B, p->ldb, p->Kw, p->Nw, Lf.n, sa, sb, kind, scale, stream));
+        p->launches += 1;
+        p->acct[0] += root_in + (double)nleaf * (double)(Lf.m * Lf.k + Lf.n * Lf.k) * pl;
         return FMM_OK;
     }
     {
         const Level& C1 = lv[1];
         View va{A, p->lda, 0, lv[0].m, lv[0].k, p->Mw, p->Kw};
-        if (p->pre16 && d == 1) {
-            Stack16 sa{p->a16[0], p->a16[1], p->ld16, C1.m * p->ld16, 7};
-            Stack16 sb{p->b16[0], p->b16[1], p->ld16, C1.n * p->ld16, 7};
-            FMM_CUDA(launch_pre_add16(va, 1, sa, 0, kind, scale, stream));
-            FMM_CUDA(launch_pre_add16_b_root(B, p->ldb, p->Kw, p->Nw, C1.k, C1.n, sb, kind, scale, stream));
-            p->acct[0] += root_in + 7.0 * (double)(C1.m * C1.k + C1.n * C1.k) * pl;
-        } else {
-            Stack sa{lv[0].achild, C1.k, C1.m * C1.k, 7};
-            FMM_CUDA(launch_pre_add(va, 1, sa, 0, 1, stream));
-            Stack sb{lv[0].bchild, C1.k, C1.n * C1.k, 7};
-            FMM_CUDA(launch_pre_add_b_root(B, p->ldb, p->Kw, p->Nw, C1.k, C1.n, sb, 1, stream));
-            p->acct[0] += root_in + 7.0 * (double)(C1.m * C1.k + C1.n * C1.k) * 4.0;
-        }
+        Stack sa{lv[0].achild, C1.k, C1.m * C1.k, 7};
+        FMM_CUDA(launch_pre_add(va, 1, sa, 0, 1, stream));
+        Stack sb{lv[0].bchild, C1.k, C1.n * C1.k, 7};
+        FMM_CUDA(launch_pre_add_b_root(B, p->ldb, p->Kw, p->Nw, C1.k, C1.n, sb, 1, stream));
+        p->acct[0] += root_in + 7.0 * (double)(C1.m * C1.k + C1.n * C1.k) * 4.0;
         p->launches += 2;
     }
     for (int l = 1; l < d; ++l) {
@@ -827,15 +819,6 @@ fmm_status_t winograd_pre(fmm_plan_s* p, const float* A, const float* B, cudaStr
             p->launches += 2;
             p->acct[0] += in + 343.0 * (double)L.nodes * (double)(Lf.m * Lf.k + Lf.n * Lf.k) * pl;
             break;
-        }
-        if (p->pre16 && l == d - 1) {
-            Stack16 sa{p->a16[0], p->a16[1], p->ld16, Ch.m * p->ld16, 7};
-            Stack16 sb{p->b16[0], p->b16[1], p->ld16, Ch.n * p->ld16, 7};
-            FMM_CUDA(launch_pre_add16(va, L.nodes, sa, 0, kind, scale, stream));
-            FMM_CUDA(launch_pre_add16(vb, L.nodes, sb, 1, kind, scale, stream));
-            p->launches += 2;
-            p->acct[0] += in + 7.0 * (double)L.nodes * (double)(Ch.m * Ch.k + Ch.n * Ch.k) * pl;
-            continue;
         }
         const int per = L.full ? 7 : 4;
         Stack sa{L.achild, Ch.k, Ch.m * Ch.k, per};

@@ -225,31 +225,26 @@ struct Stack16 {
     long long child_stride;
     int nchild;
 };
-// Pre-additions of one level writing all 7 children as split 16-bit planes
-// (the last level of a split-precision plan); scale = device {s_a, s_b} or null.
-cudaError_t launch_pre_add16(const View& parent, long long nodes, const Stack16& out, int side_b, int kind,
-                             const float* scale, cudaStream_t stream);
-cudaError_t launch_pre_add16_b_root(const float* B, long long ldb, long long K, long long N, long long kh,
-                                    long long nh, const Stack16& out, int kind, const float* scale,
-                                    cudaStream_t stream);
 // Plain split of an M x K matrix (transpose = 0) or of B^T for a K x N matrix
 // B (transpose = 1, rows = K, cols = N) into 16-bit planes; which = 0 uses
 // scale[0], 1 uses scale[1].
 cudaError_t launch_split16(const float* X, long long ldx, long long rows, long long cols, const Stack16& out,
                            int transpose, int kind, const float* scale, int which, cudaStream_t stream);
-// Two consecutive levels in one pass (middle level never stored; identical
-// arithmetic).  pre: node operands (4h x 4w, uniform stack `node`, reads
-// outside its valid window are zero) -> the 49 grandchildren as split planes
-// (child stride, ld of `out`); w must be a multiple of 4.  post: 49 grandchild
-// products per node (h x w, row stride ld_in, child stride) -> node outputs
-// (4h x 4w, row stride ld_out, node stride); valid_rows >= 0 marks the root:
-// C <- alpha * U + beta * C inside valid_rows x valid_cols.
-cudaError_t launch_pre_add2(const View& node, long long nodes, const Stack16& out, int side_b, int kind,
-                            const float* scale, cudaStream_t stream);
-// Root B side of a depth-2 plan: the caller's row-major B (K x N valid) straight
-// into the 49 leaf operands of B^T (h = N0 / 4 rows, w = K0 / 4 columns each).
-cudaError_t launch_pre_add2_b_root(const float* B, long long ldb, long long K, long long N, long long h, long long w,
-                                   const Stack16& out, int kind, const float* scale, cudaStream_t stream);
+// Pre-additions of a whole depth-1 or depth-2 recursion in one launch: the caller's
+// A (view of rows x cols padded to a multiple of 4 * 2^depth) and row-major B (valid
+// K x N) -> the 7^depth leaf operands of A and of B^T as split planes.  B^T's
+// leaves have hb rows (a multiple of 4) and A's leaf columns.
+cudaError_t launch_pre_root(int depth, const View& a, const float* B, long long ldb, long long K, long long N,
+                            long long hb, const Stack16& sa, const Stack16& sb, int kind, const float* scale,
+                            cudaStream_t stream);
+// Two consecutive levels of post-additions in one pass: 49 grandchild products per
+// node (h x w, row stride ld_in, child stride) -> node outputs (4h x 4w, row stride
+// ld_out, node stride); valid_rows >= 0 marks the root: C <- alpha * U + beta * C
+// inside valid_rows x valid_cols.
+cudaError_t launch_post_add2(const float* P, long long ld_in, long long child_stride, long long nodes, long long h,
+                             long long w, float* out, long long ld_out, long long out_node_stride,
+                             long long valid_rows, long long valid_cols, float alpha, float beta,
+                             cudaStream_t stream);
 // Root B side of a depth-3 plan straight from row-major B (valid K x N) into
 // the 343 leaf operands of B^T (h x w each, h a multiple of 4), split planes.
 cudaError_t launch_pre_add3_bt(const float* B, long long ldb, long long K, long long N, long long h, long long w,
@@ -260,10 +255,6 @@ cudaError_t launch_pre_add3_bt(const float* B, long long ldb, long long K, long 
 cudaError_t launch_pre_add3(const View& node, long long nodes, const Stack16& out, int side_b, int kind,
                             const float* scale, cudaStream_t stream);
 cudaError_t launch_post_add3(const float* P, long long ld_in, long long child_stride, long long nodes, long long h,
-                             long long w, float* out, long long ld_out, long long out_node_stride,
-                             long long valid_rows, long long valid_cols, float alpha, float beta,
-                             cudaStream_t stream);
-cudaError_t launch_post_add2(const float* P, long long ld_in, long long child_stride, long long nodes, long long h,
                              long long w, float* out, long long ld_out, long long out_node_stride,
                              long long valid_rows, long long valid_cols, float alpha, float beta,
                              cudaStream_t stream);

@@ -13,7 +13,7 @@
 // Bound: the launch, then the serial chain of K steps, each of which the L1 and
 // shared-memory pipe sets (operand loads, split stores and MMA reads; 512 loader
 // threads keep loads two steps ahead, 256 took 1.0 us a step): 0.60 / 0.65 / 0.80
-// us per 32 columns of K at tiles of 32 / 64 / 128 columns in FP32.  FP32
+// us per 32 columns of K at tiles of 32 / 64 / 128 columns in FP32.  Calls:
 // 700 x 515 x 901 45.7 us by the leaf path, 16.4 this way; 512^3 30.9 and 10.5;
 // 573 x 452 x 2103 74 and 25.
 //
