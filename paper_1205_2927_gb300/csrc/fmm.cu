@@ -550,58 +550,46 @@ SmallArgs small_args(long long M, long long N, long long K, float alpha, const f
     return a;
 }
 
-// Leaf launch over `groups` (already filled except tile bookkeeping).
-fmm_status_t run_leaves(fmm_plan_s* p, GemmArgs& args, cudaStream_t stream, int mode = -1) {
-    const bool pair = p->pair && mode < 0;   // the peel border (explicit mode) stays single-CTA
-    if (mode < 0) mode = p->mode;
-    if (pair) {
-        long long t = 0;
-        for (int g = 0; g < args.num_groups; ++g) {
-            GemmGroup& G = args.groups[g];
-            G.tiles_m = (G.M + 255) / 256;
-            G.tiles_n = (G.N + 255) / 256;
-            G.tile_begin = t;
-            t += (long long)G.tiles_m * G.tiles_n * G.batch;
-            if (mode == kLeafFP16x3P) G.scale = p->fp16_scale();
-        }
-        args.total_tiles = t;
-        args.raster_m = 16;
-        args.ext_maps = nullptr;
-        args.ext_groups = nullptr;
-        args.status = p->status;
-        if (dynamic_order(p, args)) {   // dynamic tile order: counter and rings start from zero
-            FMM_CUDA(cudaMemsetAsync(p->tile_sched, 0, kTileSchedBytes, stream));
-            args.tile_counter = reinterpret_cast<int*>(p->tile_sched);
-            args.tile_seq = reinterpret_cast<unsigned long long*>(p->tile_sched + 256);
-        }
-        args.fuse_scratch = p->fused ? p->fuse_scratch : nullptr;
-        FMM_CUDA(launch_leaf_gemm_pair(args, mode, p->num_sms, stream));
-        p->launches += args.total_tiles > 0 ? 1 : 0;
-        return FMM_OK;
-    }
+// Tile bookkeeping of a leaf launch over `groups` (already filled otherwise); under
+// the dynamic tile order the counter and rings are zeroed on `stream`.  pair: CTA-pair
+// tiles (the peel border, which has a mode of its own, stays single-CTA).
+fmm_status_t prepare_leaves(fmm_plan_s* p, GemmArgs& args, int mode, bool pair, cudaStream_t stream) {
+    const int tm = pair ? 256 : kBM, tn = pair ? 256 : p->bn;
     long long t = 0;
     for (int g = 0; g < args.num_groups; ++g) {
         GemmGroup& G = args.groups[g];
-        G.tiles_m = (G.M + kBM - 1) / kBM;
-        G.tiles_n = (G.N + p->bn - 1) / p->bn;
+        G.tiles_m = (G.M + tm - 1) / tm;
+        G.tiles_n = (G.N + tn - 1) / tn;
         G.tile_begin = t;
         t += (long long)G.tiles_m * G.tiles_n * G.batch;
+        if (mode == kLeafFP16x3 || mode == kLeafFP16x3P) G.scale = p->fp16_scale();
     }
     args.total_tiles = t;
     args.raster_m = 16;
     args.ext_maps = nullptr;
     args.ext_groups = nullptr;
+    args.status = p->status;
     if (dynamic_order(p, args)) {   // dynamic tile order: counter and rings start from zero
         FMM_CUDA(cudaMemsetAsync(p->tile_sched, 0, kTileSchedBytes, stream));
         args.tile_counter = reinterpret_cast<int*>(p->tile_sched);
         args.tile_seq = reinterpret_cast<unsigned long long*>(p->tile_sched + 256);
     }
-    if (mode == kLeafFP16x3 || mode == kLeafFP16x3P)
-        for (int g = 0; g < args.num_groups; ++g) args.groups[g].scale = p->fp16_scale();
-    args.status = p->status;
-    FMM_CUDA(launch_leaf_gemm(args, mode, p->bn, p->num_sms, stream));
+    if (pair) args.fuse_scratch = p->fused ? p->fuse_scratch : nullptr;
+    return FMM_OK;
+}
+
+fmm_status_t launch_leaves(fmm_plan_s* p, const GemmArgs& args, int mode, bool pair, cudaStream_t stream) {
+    if (pair) FMM_CUDA(launch_leaf_gemm_pair(args, mode, p->num_sms, stream));
+    else FMM_CUDA(launch_leaf_gemm(args, mode, p->bn, p->num_sms, stream));
     p->launches += args.total_tiles > 0 ? 1 : 0;
     return FMM_OK;
+}
+
+fmm_status_t run_leaves(fmm_plan_s* p, GemmArgs& args, cudaStream_t stream, int mode = -1) {
+    const bool pair = p->pair && mode < 0;
+    if (mode < 0) mode = p->mode;
+    const fmm_status_t s = prepare_leaves(p, args, mode, pair, stream);
+    return s != FMM_OK ? s : launch_leaves(p, args, mode, pair, stream);
 }
 
 // K chunks of the classical recursion of Table 1 (RMUL) at depth d: every level
@@ -992,16 +980,17 @@ fmm_status_t run_winograd(fmm_plan_s* p, float alpha, const float* A, const floa
                           cudaStream_t stream) {
     p->border_beta = beta;
     fmm_status_t s;
+    // the leaf launch's tables and counters first: nothing then stands between the
+    // passes, and each launch overlaps the end of the one before it
+    GemmArgs args;
+    memset(&args, 0, sizeof(args));
+    int nm = 0, ng = 0;
+    if ((s = winograd_leaf_groups(p, args.maps, nm, args.groups, ng)) != FMM_OK) return s;
+    args.num_groups = ng;
+    if ((s = prepare_leaves(p, args, p->mode, p->pair != 0, stream)) != FMM_OK) return s;
     if ((s = winograd_pre(p, A, B, stream)) != FMM_OK) return s;
     mark(p, 1, stream);
-    {
-        GemmArgs args;
-        memset(&args, 0, sizeof(args));
-        int nm = 0, ng = 0;
-        if ((s = winograd_leaf_groups(p, args.maps, nm, args.groups, ng)) != FMM_OK) return s;
-        args.num_groups = ng;
-        if ((s = run_leaves(p, args, stream)) != FMM_OK) return s;
-    }
+    if ((s = launch_leaves(p, args, p->mode, p->pair != 0, stream)) != FMM_OK) return s;
     mark(p, 2, stream);
     if ((s = winograd_post(p, alpha, beta, C, stream)) != FMM_OK) return s;
     if (p->peel && (p->Mw < p->M || p->Kw < p->K || p->Nw < p->N)) return run_border(p, alpha, A, B, C, stream);
@@ -1406,13 +1395,13 @@ void make_tmp(fmm_plan_s& t, long long M, long long N, long long K, long long ld
             t.split_kind = kSplitTF32X;
         }
     }
-    // depth 0 with the leaf tile left open: small products in one launch where the
-    // models favour it.  Planners that time tiles reach it by their 256 candidate;
-    // a caller who fixes depth 0 for leaves of 1024 and more keeps the leaf path,
-    // whose operand passes fmm_plan_phase_bytes reports
+    // depth 0, by whichever planner, with the leaf tile left open: small products in
+    // one launch where the models favour it.  A caller who fixes depth 0 for leaves of
+    // 1024 and more keeps the leaf path, whose operand passes fmm_plan_phase_bytes
+    // reports
     t.small_bn = 0;
     if (!t.host && outer == 0 && t.depth == 0 && t.rmul == 0 && o.leaf_tile == 0 && M > 0 && N > 0 && K > 0 &&
-        (o.planner == FMM_PLANNER_FIXED || bn == 256) && (std::min(M, N) < 1024 || o.depth < 0))
+        (std::min(M, N) < 1024 || o.depth < 0))
         t.small_bn = small_choice(M, N, K, lda, o.precision, bn == 512, 1, true, &t.small_splits);
     // the fused last level needs the CTA-pair kernel on split planes and a
     // Winograd depth of 2 to 4 (the node outputs then fold into C in one pass)
@@ -1679,10 +1668,7 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
 
 // Score the candidates with the registered network (one inference launch) and
 // return the index of the smallest predicted time (ties: smaller depth, then
-// the larger tile).  The fixed rule's plan is kept unless that is predicted to
-// take a fifth less: predictions miss by several percent (more where tiles
-// quantise), and the fixed rule is within 1 % of the best candidate over 60
-// unseen shapes.
+// the larger tile).
 fmm_status_t choose_mlp(long long M, long long N, long long K, const fmm_options_t& o, const Cand* c, int n,
                         int* best, cudaStream_t stream) {
     int dev = 0;
@@ -1715,9 +1701,6 @@ fmm_status_t choose_mlp(long long M, long long N, long long K, const fmm_options
         if (d < -1e-6f) b = i;
         else if (d <= 1e-6f && (c[i].depth < c[b].depth || (c[i].depth == c[b].depth && c[i].bn > c[b].bn))) b = i;
     }
-    const int fixed = fixed_depth(M, N, K, o.cutoff), tile = o.leaf_tile ? o.leaf_tile : auto_tile(M, N, fixed, o);
-    for (int i = 0; i < n; ++i)   // outputs are log(ms)
-        if (c[i].depth == fixed && c[i].bn == tile && Y[b] > Y[i] - 0.223f) b = i;
     *best = b;
     return FMM_OK;
 }
@@ -1737,7 +1720,7 @@ fmm_status_t autotune_core(long long M, long long N, long long K, const fmm_opti
         fmm_plan_s t;
         fmm_options_t od = o;
         od.host_operands = 0;   // candidates are timed on device operands
-        od.planner = FMM_PLANNER_EXHAUSTIVE;   // each tile as itself (make_tmp)
+        od.leaf_tile = c[i].bn;   // leaf tiles as themselves (make_tmp's small products have none)
         make_tmp(t, M, N, K, K, N, N, od, c[i].depth, c[i].bn);
         size_t need = 0;
         layout(&t, nullptr, &need);

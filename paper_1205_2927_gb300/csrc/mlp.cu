@@ -10,6 +10,7 @@
 // blocks' sums added in a fixed order and Adam in place.
 #include "../../include/fmm.h"
 #include "fmm_internal.h"
+#include "ptx.cuh"
 
 namespace fmm {
 namespace {
@@ -119,6 +120,7 @@ __global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* __restric
                                                           int per, float* __restrict__ rows, AdamArgs a) {
     extern __shared__ float4 train_smem[];
     TrainSmem& S = *reinterpret_cast<TrainSmem*>(train_smem);
+    dep_start();
     const int t = threadIdx.x, sg = t & 7, ug = t >> 3;      // samples sg + 8 q; units ug + 16 u, or 4 ug + u
     const int u0 = 4 * ug;
     const int i8 = 8 * (t & 7), j4 = 4 * (t >> 3);           // dW2 rows i8 .. + 7, columns j4 .. + 3
@@ -299,6 +301,7 @@ __global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* __restric
 // place.
 __global__ void __launch_bounds__(512) mlp_adam_kernel(const float* __restrict__ rows, int nrows, AdamArgs a) {
     __shared__ float part[16][32];
+    dep_start();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
     float g = 0.f;
     if (p <= NPARAM) {
@@ -363,10 +366,10 @@ extern "C" fmm_status_t fmm_mlp_train_step(float* params, float* adam_m, float* 
     }
     float* rows = static_cast<float*>(workspace);
     if (blocks == 1) {
-        mlp_train_kernel<true><<<1, NT, sizeof(TrainSmem), s>>>(X, T, tiles_per, nullptr, a);
+        launch_dep(mlp_train_kernel<true>, 1, NT, sizeof(TrainSmem), s, X, T, tiles_per, nullptr, a);
     } else {
-        mlp_train_kernel<false><<<blocks, NT, sizeof(TrainSmem), s>>>(X, T, tiles_per, rows, a);
-        mlp_adam_kernel<<<(ROW + 31) / 32, 512, 0, s>>>(rows, blocks, a);
+        launch_dep(mlp_train_kernel<false>, blocks, NT, sizeof(TrainSmem), s, X, T, tiles_per, rows, a);
+        launch_dep(mlp_adam_kernel, (ROW + 31) / 32, 512, 0, s, rows, blocks, a);
     }
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }

@@ -25,6 +25,20 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
+// Kernels launched by launch_dep.  dep_wait: until the kernel before this one has
+// completed and its writes are visible.  dep_trigger: once every block has called it
+// (or ended), the next such kernel's blocks may become resident.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Both, at the start of a short kernel (not of kernels of very many short blocks:
+// 350,000 blocks of a batched copy paid 5 % for the two instructions).  The persistent leaf kernels trigger when a
+// block has issued its last tile: blocks that waited beside them from the start
+// slowed 512 uneven products from 6.85 to 7.22 ms.
+__device__ __forceinline__ void dep_start() {
+    dep_trigger();
+    dep_wait();
+}
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");

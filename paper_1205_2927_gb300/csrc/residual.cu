@@ -8,6 +8,7 @@
 // pass over A, B and C: bandwidth-bound in fp32.
 #include "../../include/fmm.h"
 #include "fmm_internal.h"
+#include "ptx.cuh"
 
 #include <cstdint>
 #include <type_traits>
@@ -28,6 +29,7 @@ __global__ void __launch_bounds__(256) rowdot_kernel(const float* __restrict__ X
                                                      Out* __restrict__ out, const double* __restrict__ sub,
                                                      int vec4) {
     __shared__ Acc warp_sum[8];
+    dep_start();
     const long long row = blockIdx.x;
     const int t = threadIdx.x;
     const float* xr = X + row * ld;
@@ -112,6 +114,7 @@ __global__ void __launch_bounds__(256, 3) rowdot64_kernel(const float* __restric
                                                                      double* __restrict__ out,
                                                                      const double* __restrict__ sub) {
     __shared__ double warp_sum[8][R];
+    dep_start();
     const long long row0 = (long long)blockIdx.x * R;
     const int t = threadIdx.x, nr = rows - row0 < R ? (int)(rows - row0) : R;
     const float* xr[R];
@@ -187,11 +190,11 @@ void rowdot64(const float* X, long long ld, long long rows, long long cols, cons
     const bool wide = rows >= 304LL * R;
     const unsigned grid = (unsigned)(wide ? (rows + R - 1) / R : rows);
     if (vec4) {
-        if (wide) rowdot64_kernel<Vec, 4, true><<<grid, 256, 0, s>>>(X, ld, rows, cols, v, out, sub);
-        else rowdot64_kernel<Vec, 1, true><<<grid, 256, 0, s>>>(X, ld, rows, cols, v, out, sub);
+        if (wide) launch_dep(rowdot64_kernel<Vec, 4, true>, grid, 256, 0, s, X, ld, rows, cols, v, out, sub);
+        else launch_dep(rowdot64_kernel<Vec, 1, true>, grid, 256, 0, s, X, ld, rows, cols, v, out, sub);
     } else {
-        if (wide) rowdot64_kernel<Vec, 8, false><<<grid, 256, 0, s>>>(X, ld, rows, cols, v, out, sub);
-        else rowdot64_kernel<Vec, 1, false><<<grid, 256, 0, s>>>(X, ld, rows, cols, v, out, sub);
+        if (wide) launch_dep(rowdot64_kernel<Vec, 8, false>, grid, 256, 0, s, X, ld, rows, cols, v, out, sub);
+        else launch_dep(rowdot64_kernel<Vec, 1, false>, grid, 256, 0, s, X, ld, rows, cols, v, out, sub);
     }
 }
 
@@ -213,9 +216,9 @@ cudaError_t residual_impl(long long M, long long N, long long K, const float* A,
         rowdot64<double>(A, lda, M, K, y, z, nullptr, av, s);
         rowdot64<float>(C, ldc, M, N, x, r, z, cv, s);
     } else {
-        if (K > 0) rowdot_kernel<Acc, float, Acc><<<(unsigned)K, 256, 0, s>>>(B, ldb, K, N, x, y, nullptr, bv);
-        rowdot_kernel<Acc, Acc, double><<<(unsigned)M, 256, 0, s>>>(A, lda, M, K, y, z, nullptr, av);
-        rowdot_kernel<Acc, float, double><<<(unsigned)M, 256, 0, s>>>(C, ldc, M, N, x, r, z, cv);
+        if (K > 0) launch_dep(rowdot_kernel<Acc, float, Acc>, (unsigned)K, 256, 0, s, B, ldb, K, N, x, y, nullptr, bv);
+        launch_dep(rowdot_kernel<Acc, Acc, double>, (unsigned)M, 256, 0, s, A, lda, M, K, y, z, nullptr, av);
+        launch_dep(rowdot_kernel<Acc, float, double>, (unsigned)M, 256, 0, s, C, ldc, M, N, x, r, z, cv);
     }
     return cudaGetLastError();
 }

@@ -130,9 +130,6 @@ __global__ void __launch_bounds__(544, 1) small_gemm_kernel(const SmallArgs args
     unsigned* status = args.status;
 
     if (t == 0) {
-        // a call that owns its status word starts it from zero: waits run out, and
-        // report, seconds after the launch's first block has passed here
-        if (args.clear_status && blockIdx.x == 0) *status = 0u;
         for (int s = 0; s < Cfg::kStages; ++s) {
             mbar_init(full_bar(s), NL / 32);   // one arrival per loader warp
             mbar_init(empty_bar(s), 1);
@@ -149,6 +146,10 @@ __global__ void __launch_bounds__(544, 1) small_gemm_kernel(const SmallArgs args
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    dep_start();
+    // a call that owns its status word starts it from zero: waits run out, and
+    // report, seconds after the launch's first block has passed here
+    if (args.clear_status && blockIdx.x == 0 && t == 0) *status = 0u;
     bool ok = true;
 
     if (warp < NL / 32) {
@@ -348,16 +349,18 @@ cudaError_t launch(const SmallArgs& a, cudaStream_t stream) {
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
     }
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = (unsigned)a.splits;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)a.splits;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_dep
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3((unsigned)((long long)a.tiles_m * a.tiles_n * a.splits));
     cfg.blockDim = dim3(Cfg::kLoaders + 32);
     cfg.dynamicSmemBytes = Cfg::kSmem;
     cfg.stream = stream;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
