@@ -467,14 +467,22 @@ int fixed_depth(long long M, long long N, long long K, int cutoff) {
     return d;
 }
 
-// Leaf tile when the caller leaves it open: the CTA-pair 256 x 256 tile once
-// both output sides of every leaf reach 1024 (from there on it is at least as
-// fast as the single-CTA tile and cuts the per-SM operand traffic by a third),
-// the single-CTA 128 x 256 tile otherwise.
-int auto_tile(long long M, long long N, int depth, const fmm_options_t& o) {
-    (void)o;
+// Leaf tile when the caller leaves it open.  Recursive plans: the CTA-pair 256 x 256
+// tile once both output sides of every leaf reach 1024 (from there on it is at
+// least as fast as the single-CTA tile and cuts the per-SM operand traffic by a
+// third).  Depth 0: the pair tile on long K (below outputs of 1024 it gains FP32 4 to
+// 37 % from K = 460 on, TF32 up to 36 % from 1000, the 16-bit splits 0 to 7 % from
+// 2000, over 78 shapes of 256 .. 8192) unless its waves of 76 pairs, at `rel` of a
+// single-CTA wave's time each, take longer than the 128 x 256 tile's of 152 SMs
+// (583 x 7585 x 726, 2 waves against 1: 56 us against 47).
+int auto_tile(long long M, long long N, long long K, int depth, const fmm_options_t& o) {
     const long long mn = M < N ? M : N;
-    return (mn >> depth) >= 1024 ? 512 : 256;
+    if (depth > 0) return (mn >> depth) >= 1024 ? 512 : 256;
+    const bool fp32 = o.precision == FMM_PREC_FP32, tf32 = o.precision == FMM_PREC_TF32;
+    if (mn < 1024 && (mn <= 256 || K < (fp32 ? 384 : tf32 ? 1024 : 2048))) return 256;
+    const long long pair = ((M + 255) / 256) * ((N + 255) / 256), single = ((M + 127) / 128) * ((N + 255) / 256);
+    const double rel = fp32 ? (tf32x_leaf(K, 0) ? 0.65 : 0.9) : tf32 ? 0.82 : 1.0;
+    return (double)((pair + 75) / 76) * rel <= (double)((single + 151) / 152) ? 512 : 256;
 }
 
 // Whether a leaf launch takes its tiles in dynamic order: launches over several
@@ -521,7 +529,7 @@ int small_choice(long long M, long long N, long long K, long long lda, fmm_preci
                 continue;
             const double resident = sp == 8 ? 128.0 : sp == 4 ? 144.0 : 152.0;   // CTAs whose clusters fit at once
             const double steps = std::ceil(std::ceil((double)K / 32.0) / sp);
-            const double c = m.c[i] * (lda % 4 ? 1.2 : 1.0);   // rows off the 16-byte grid load by 4 bytes
+            const double c = m.c[i] * (lda % 4 ? 1.5 : 1.0);   // rows off the 16-byte grid load by 4 bytes
             const double t = 7.0 + std::ceil(tiles * sp / resident) * (2.0 + steps * c);
             if (t < best) {
                 best = t;
@@ -535,7 +543,8 @@ int small_choice(long long M, long long N, long long K, long long lda, fmm_preci
     const double waves = std::ceil(std::ceil((double)M / tm) * std::ceil((double)N / 256.0) / slots);
     const double leaf = m.launches + ((double)M * K * m.a_bytes + (double)K * N * m.b_bytes) / 6e6 +
                         waves * (4.0 + (double)K * (pair ? m.k_pair : m.k));
-    return best < 0.85 * leaf ? best_bn : 0;   // the models miss by up to 15 %
+    // the models miss by up to 15 % on long K, where operands come from DRAM
+    return best < (K <= 4096 ? 0.97 : 0.85) * leaf ? best_bn : 0;
 }
 
 SmallArgs small_args(long long M, long long N, long long K, float alpha, const float* A, long long lda, const float* B,
@@ -1759,11 +1768,11 @@ fmm_status_t plan_choose(long long M, long long N, long long K, long long lda, l
     if (o.planner == FMM_PLANNER_FIXED || o.algo == FMM_ALGO_CLASSICAL || M == 0 || N == 0 || K == 0) {
         depth = o.depth >= 0 ? o.depth : fixed_depth(M, N, K, o.cutoff);
         if (o.algo == FMM_ALGO_CLASSICAL) {   // one launch spans all of C: tile by M, N
-            bn = o.leaf_tile ? o.leaf_tile : auto_tile(M, N, 0, o);
+            bn = o.leaf_tile ? o.leaf_tile : auto_tile(M, N, K, 0, o);
             *need = plan_bytes(M, N, K, lda, ldb, ldc, o, depth, bn);
             return FMM_OK;
         }
-        bn = o.leaf_tile ? o.leaf_tile : auto_tile(M, N, depth, o);
+        bn = o.leaf_tile ? o.leaf_tile : auto_tile(M, N, K, depth, o);
         *need = plan_bytes(M, N, K, lda, ldb, ldc, o, depth, bn);
         return FMM_OK;
     }
