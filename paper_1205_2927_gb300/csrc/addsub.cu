@@ -303,41 +303,64 @@ __global__ void fill_kernel(float* p, size_t n, unsigned seed) {
     }
 }
 
-// max |x| over a rows x cols matrix, folded into *out (float bits; non-negative
-// floats order like unsigned integers)
-// max |X| over a rows x cols operand (row stride ld): rows grid-strided over
-// blockIdx.y, columns over blockIdx.x; 16-byte loads when the rows allow;
-// one atomic per block.
-__global__ void __launch_bounds__(256) absmax_kernel(const float* __restrict__ X, long long ld, long long rows,
-                                                     long long cols, unsigned* out) {
-    dep_start();
-    __shared__ float warp_max[8];
-    const bool vec = (reinterpret_cast<uintptr_t>(X) & 15) == 0 && (ld & 3) == 0;
-    const long long step = (long long)gridDim.x * blockDim.x;
-    float m = 0.f;
-    for (long long r = blockIdx.y; r < rows; r += gridDim.y) {
-        const float* xr = X + r * ld;
-        if (vec) {
-            const long long groups = cols >> 2;
-            for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < groups; g += step) {
-                const float4 v = __ldg(reinterpret_cast<const float4*>(xr) + g);
-                m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
-            }
-            for (long long c = (groups << 2) + (long long)blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += step)
-                m = fmaxf(m, fabsf(__ldg(xr + c)));
+// max |x| of A and of B in one launch, folded into mx[0] and mx[1] (float bits;
+// non-negative floats order like unsigned integers).  Blocks stride over 32 x 128
+// blocks of both operands, two at a time: eight 16-byte loads per thread in
+// flight where the rows allow; one atomic per block and operand.  Bound: HBM.
+// n = 8192: 78 us, against 70 + 70 for one launch per operand with two loads
+// in flight.
+struct MaxOperand {
+    const float* X;
+    long long ld, rows, cols, tiles_c, tiles;   // tiles_c 128-column blocks per 32-row band
+};
+__device__ __forceinline__ void absmax_load(const MaxOperand& o, bool vec, long long tile, int tid, float4 (&v)[4]) {
+    const long long band = tile / o.tiles_c, r0 = band * 32, c0 = (tile - band * o.tiles_c) * 128;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int g = tid + 256 * j;   // row g / 32 of the block, columns 4 (g % 32) .. + 3
+        const long long r = r0 + (g >> 5), c = c0 + 4 * (g & 31);
+        v[j] = f4(0.f, 0.f, 0.f, 0.f);
+        if (r >= o.rows || c >= o.cols) continue;
+        const float* src = o.X + r * o.ld + c;
+        if (vec && c + 3 < o.cols) {
+            v[j] = __ldg(reinterpret_cast<const float4*>(src));
         } else {
-            for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += step)
-                m = fmaxf(m, fabsf(__ldg(xr + c)));
+            v[j].x = __ldg(src);
+            if (c + 1 < o.cols) v[j].y = __ldg(src + 1);
+            if (c + 2 < o.cols) v[j].z = __ldg(src + 2);
+            if (c + 3 < o.cols) v[j].w = __ldg(src + 3);
         }
     }
+}
+__global__ void __launch_bounds__(256) absmax_kernel(MaxOperand A, MaxOperand B, unsigned* mx) {
+    __shared__ float warp_max[8];
+    dep_start();
+    const int tid = threadIdx.x;
+#pragma unroll 1
+    for (int which = 0; which < 2; ++which) {
+        const MaxOperand& o = which ? B : A;
+        const bool vec = (reinterpret_cast<uintptr_t>(o.X) & 15) == 0 && (o.ld & 3) == 0;
+        float m = 0.f;
+        for (long long t = blockIdx.x; t < o.tiles; t += 2LL * gridDim.x) {
+            float4 v[2][4];
+            absmax_load(o, vec, t, tid, v[0]);
+            absmax_load(o, vec, min(t + gridDim.x, o.tiles - 1), tid, v[1]);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
+            for (int i = 0; i < 8; ++i) {
+                const float4 x = v[i >> 2][i & 3];
+                m = fmaxf(fmaxf(m, fmaxf(fabsf(x.x), fabsf(x.y))), fmaxf(fabsf(x.z), fabsf(x.w)));
+            }
+        }
 #pragma unroll
-        for (int w = 1; w < 8; ++w) m = fmaxf(m, warp_max[w]);
-        atomicMax(out, __float_as_uint(m));
+        for (int s = 16; s > 0; s >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, s));
+        if ((tid & 31) == 0) warp_max[tid >> 5] = m;
+        __syncthreads();
+        if (tid == 0) {
+#pragma unroll
+            for (int w = 1; w < 8; ++w) m = fmaxf(m, warp_max[w]);
+            if (blockIdx.x < o.tiles) atomicMax(mx + which, __float_as_uint(m));
+        }
+        __syncthreads();
     }
 }
 
@@ -708,9 +731,10 @@ __device__ __forceinline__ void emit_children(const float4 (&X)[1 << D][1 << D],
 //     bytes in shared memory (every load before the first store; 17 floats a row:
 //     the reads are free of bank conflicts) and then, like an A thread, holds 4
 //     consecutive k of one n and stores along k.
-// Bound: HBM.  n = 8192, depth 2, FP32: both sides PRE2_US us (1.91 GB each way of
-// 2.0), against 284 + 334 us for one launch per side whose B pass turned each
-// group of seven outputs through shared memory; n = 1024: 8.3 + 15.4 -> PRE1K_US us.
+// Bound: HBM writes.  n = 8192, depth 2, FP32: both sides 606 us (3.83 GB, 3.29 of
+// them written: 6.3 TB/s), against 284 + 334 us for one launch per side whose B pass
+// turned each group of seven outputs through shared memory; n = 4096, depth 1: 43 +
+// 49 -> 86 us; n = 1024, depth 2: 8.3 + 15.4 -> 11.5 us.
 constexpr int kRootN = 16, kRootK = 32, kRootPitch = kRootN + 1;
 struct RootB {
     const float* ptr;
@@ -1285,8 +1309,14 @@ cudaError_t launch_fp16_scales(const float* A, long long lda, long long M, long 
                                cudaStream_t stream) {
     cudaError_t e = cudaMemsetAsync(scratch, 0, 2 * sizeof(unsigned), stream);
     if (e != cudaSuccess) return e;
-    if (M > 0 && K > 0) launch_dep(absmax_kernel, dim3(4, gy(M < 1024 ? M : 1024)), 256, 0, stream, A, lda, M, K, scratch);
-    if (K > 0 && N > 0) launch_dep(absmax_kernel, dim3(4, gy(K < 1024 ? K : 1024)), 256, 0, stream, B, ldb, K, N, scratch + 1);
+    auto operand = [](const float* X, long long ld, long long rows, long long cols) {
+        const long long tc = (cols + 127) / 128;
+        return MaxOperand{X, ld, rows, cols, tc > 0 ? tc : 1, tc * ((rows + 31) / 32)};
+    };
+    const MaxOperand a = operand(A, lda, M, K), b = operand(B, ldb, K, N);
+    const long long most = (a.tiles > b.tiles ? a.tiles : b.tiles);
+    const long long grid = (most + 1) / 2 < 152 * 8 ? (most + 1) / 2 : 152 * 8;
+    if (grid > 0) absmax_kernel<<<(unsigned)grid, 256, 0, stream>>>(a, b, scratch);
     launch_dep(fp16_scale_kernel, 1, 32, 0, stream, scratch, bound_mult, scale);
     return cudaGetLastError();
 }
