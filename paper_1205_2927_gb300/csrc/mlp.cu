@@ -62,8 +62,10 @@ __global__ void __launch_bounds__(128) mlp_forward_kernel(const float* __restric
 // fixed order, so a step is deterministic.
 //
 // Bound: latency of a few warps of fp32 arithmetic per SM (batch 20000: 0.25
-// GFMA).  One thread per parameter summing the whole batch in series, on 37
-// blocks, took 1066 us a step at batch 20000; this takes 37 us.
+// GFMA), shared-memory reads next (L1 71 %).  One thread per parameter summing the
+// whole batch in series, on 37 blocks, took 1066 us a step at batch 20000; this takes
+// 32.0 us (33.4 with one multiply-add per instruction; four blocks per SM, whose
+// registers no longer hold a tile's outputs and gradients: 32.6).
 constexpr int TS = 32, NT = 128;   // samples per tile, threads per block
 constexpr int PU = HID + 4;        // row pitch (floats)
 struct TrainSmem {
@@ -106,6 +108,18 @@ __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast
 __device__ __forceinline__ void st4(float* p, float a, float b, float c, float d) {
     *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
 }
+// Two fp32 multiply-adds in one instruction, each rounded as fmaf rounds: half the
+// issue slots of the products.
+struct f2 { unsigned long long v; };
+__device__ __forceinline__ f2 pack2(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f2 x, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v)); }
+__device__ __forceinline__ void fma2(f2& acc, f2 a, f2 b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc.v) : "l"(a.v), "l"(b.v));
+}
 __device__ __forceinline__ float sum8(float x) {   // over the eight sample groups of a unit group
     x += __shfl_xor_sync(0xffffffffu, x, 1);
     x += __shfl_xor_sync(0xffffffffu, x, 2);
@@ -138,7 +152,8 @@ __global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* __restric
         S.w3[t] = a.params[OFF_W3 + t];
     }
     if (t == 0) S.b3 = a.params[OFF_B3];
-    float gw2[8][4] = {}, gb1[4] = {}, gb2[4] = {}, gw3[4] = {}, gw1[3] = {}, gb3 = 0.f, sq = 0.f;
+    f2 gw2[8][2] = {};
+    float gb1[4] = {}, gb2[4] = {}, gw3[4] = {}, gw1[3] = {}, gb3 = 0.f, sq = 0.f;
     const int tiles = (a.batch + TS - 1) / TS;
     for (int tile = blockIdx.x * per; tile < min(tiles, (int)(blockIdx.x + 1) * per); ++tile) {
         const int base = tile * TS, valid = min(TS, a.batch - base);
@@ -160,11 +175,11 @@ __global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* __restric
             st4(&S.h1[row][u0], h[0], h[1], h[2], h[3]);
         }
         __syncthreads();
-        float z[4][4];   // [sample sg + 8 q][unit ug + 16 u]
+        f2 z2[4][4];     // sums over even and odd j
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int u = 0; u < 4; ++u) z[q][u] = S.b2[ug + 16 * u];
+            for (int u = 0; u < 4; ++u) z2[q][u] = pack2(S.b2[ug + 16 * u], 0.f);
 #pragma unroll 2
         for (int j = 0; j < HID; j += 4) {
             float4 h[4], w[4];
@@ -176,12 +191,19 @@ __global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* __restric
             for (int q = 0; q < 4; ++q)
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    z[q][u] += h[q].x * w[u].x;
-                    z[q][u] += h[q].y * w[u].y;
-                    z[q][u] += h[q].z * w[u].z;
-                    z[q][u] += h[q].w * w[u].w;
+                    fma2(z2[q][u], pack2(h[q].x, h[q].y), pack2(w[u].x, w[u].y));
+                    fma2(z2[q][u], pack2(h[q].z, h[q].w), pack2(w[u].z, w[u].w));
                 }
         }
+        float z[4][4];   // [sample sg + 8 q][unit ug + 16 u]
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                float a0, a1;
+                unpack2(z2[q][u], a0, a1);
+                z[q][u] = a0 + a1;
+            }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             float y = 0.f;
@@ -216,7 +238,7 @@ __global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* __restric
             }
         }
         __syncthreads();
-        float dh[4][4] = {};   // [sample sg + 8 q][unit 4 ug + u]
+        f2 dh2[4][2] = {};     // [sample sg + 8 q][units 4 ug + 2 p, + 1]
 #pragma unroll 2
         for (int i = 0; i < HID; i += 4) {
             float4 d[4], w[4];
@@ -229,12 +251,17 @@ __global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* __restric
                 const float dd[4] = {d[q].x, d[q].y, d[q].z, d[q].w};
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    dh[q][0] += dd[k] * w[k].x;
-                    dh[q][1] += dd[k] * w[k].y;
-                    dh[q][2] += dd[k] * w[k].z;
-                    dh[q][3] += dd[k] * w[k].w;
+                    const f2 x = pack2(dd[k], dd[k]);
+                    fma2(dh2[q][0], x, pack2(w[k].x, w[k].y));
+                    fma2(dh2[q][1], x, pack2(w[k].z, w[k].w));
                 }
             }
+        }
+        float dh[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            unpack2(dh2[q][0], dh[q][0], dh[q][1]);
+            unpack2(dh2[q][1], dh[q][2], dh[q][3]);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -250,11 +277,14 @@ __global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* __restric
 #pragma unroll 2
         for (int q = 0; q < TS; ++q) {   // dW2 += dz2^T h1
             const float4 d0 = ld4(&S.dz2[q][i8]), d1 = ld4(&S.dz2[q][i8 + 4]), h = ld4(&S.h1[q][j4]);
-            const float dd[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w}, hh[4] = {h.x, h.y, h.z, h.w};
+            const float dd[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+            const f2 h01 = pack2(h.x, h.y), h23 = pack2(h.z, h.w);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) gw2[i][j] += dd[i] * hh[j];
+            for (int i = 0; i < 8; ++i) {
+                const f2 x = pack2(dd[i], dd[i]);
+                fma2(gw2[i][0], x, h01);
+                fma2(gw2[i][1], x, h23);
+            }
         }
         __syncthreads();
 #pragma unroll
@@ -271,7 +301,12 @@ __global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* __restric
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) emit(OFF_W2 + (i8 + i) * HID + j4 + j, gw2[i][j]);
+        for (int j = 0; j < 2; ++j) {
+            float g0, g1;
+            unpack2(gw2[i][j], g0, g1);
+            emit(OFF_W2 + (i8 + i) * HID + j4 + 2 * j, g0);
+            emit(OFF_W2 + (i8 + i) * HID + j4 + 2 * j + 1, g1);
+        }
 #pragma unroll
     for (int e = 0; e < 3; ++e) emit(OFF_W1 + t + e * NT, gw1[e]);
 #pragma unroll
