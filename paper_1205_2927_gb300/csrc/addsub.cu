@@ -832,15 +832,6 @@ __device__ __forceinline__ float child_of1(int i, float Q0, float Q1, float Q2, 
 // One value into the planes at element offset o (evict-first stores).
 template <int KIND>
 __device__ __forceinline__ void split_store1(void* hi_plane, void* lo_plane, long long o, float v, float sc) {
-    if constexpr (KIND == kSplitTF32X) {
-        const float hv = tf32_round_hi(v);
-        const uint32_t p = bf16x2_sat(hv, v - hv);
-        unsigned short* hl = static_cast<unsigned short*>(lo_plane) + tf32x_off(o);
-        __stcs(static_cast<float*>(hi_plane) + o, hv);
-        __stcs(hl, (unsigned short)(p & 0xffffu));
-        __stcs(hl + 32, (unsigned short)(p >> 16));
-        return;
-    }
     if constexpr (KIND == kSplitTF32) {
         __stcs(static_cast<float*>(hi_plane) + o, v);
         __stcs(static_cast<float*>(lo_plane) + o, tf32_round_rne(v - tf32_trunc(v)));
@@ -876,8 +867,7 @@ __global__ void __launch_bounds__(256, 2) pre_add3_kernel(View P, long long h, l
                                                        const float* __restrict__ scale) {
     dep_start();
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= plane_cols<KIND>(w)) return;
-    if (c >= w) P.valid_rows = 0;   // padding columns of a tf32x plane: zeros
+    if (c >= w) return;
     const float sc = scale ? scale[SIDE_B] : 1.0f;
     const long long node = blockIdx.z;
     const float* base = P.ptr + node * P.node_stride;
@@ -969,7 +959,7 @@ __global__ void __launch_bounds__(256, 2) pre_add3_bt_kernel(const float* __rest
     __syncthreads();
     const int tn = t >> 5, tk = t & 31;
     const long long n = n0 + tn, k = k0 + tk;
-    if (n >= h || k >= plane_cols<KIND>(w)) return;
+    if (n >= h || k >= w) return;
     float X[8][8];   // sub-block (a, b) of B^T at position (n, k)
 #pragma unroll
     for (int a = 0; a < 8; ++a)
@@ -1406,7 +1396,6 @@ cudaError_t launch_pre_add3(const View& node, long long nodes, const Stack16& ou
     switch (kind) {                                          \
         case kSplitBF16: FMM_PRE3(S, kSplitBF16); break;    \
         case kSplitFP16: FMM_PRE3(S, kSplitFP16); break;    \
-        case kSplitTF32X: FMM_PRE3(S, kSplitTF32X); break;  \
         default: FMM_PRE3(S, kSplitTF32); break;            \
     }
     if (side_b) { FMM_PRE3K(1) } else { FMM_PRE3K(0) }
@@ -1441,7 +1430,6 @@ cudaError_t launch_pre_add3_bt(const float* B, long long ldb, long long K, long 
     switch (kind) {
         case kSplitBF16: return launch_pre_add3_bt_impl<kSplitBF16>(B, ldb, K, N, h, w, out, scale, stream);
         case kSplitFP16: return launch_pre_add3_bt_impl<kSplitFP16>(B, ldb, K, N, h, w, out, scale, stream);
-        case kSplitTF32X: return launch_pre_add3_bt_impl<kSplitTF32X>(B, ldb, K, N, h, w, out, scale, stream);
         default: return launch_pre_add3_bt_impl<kSplitTF32>(B, ldb, K, N, h, w, out, scale, stream);
     }
 }
