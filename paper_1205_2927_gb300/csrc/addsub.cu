@@ -437,29 +437,35 @@ __global__ void batched_fp16_scale_kernel(const unsigned* __restrict__ maxima, c
 }
 
 // Root pre-additions of the host-streamed schedule: the four quadrants are
-// separate row-major buffers (h x w, row stride ld); writes the four sums.
-//   A side: S1 = Q2 + Q3, S2 = S1 - Q0, S3 = Q0 - Q2, S4 = Q1 - S2
-//   B side: T1 = Q1 - Q0, T2 = Q3 - T1, T3 = Q3 - Q1, T4 = T2 - Q2
-template <int SIDE_B>
+// separate row-major buffers (h x w, row stride ld), and a launch forms the sums
+// whose quadrants have arrived.
+//   A side: S1 = Q2 + Q3, S2 = S1 - Q0, S3 = Q0 - Q2, then S4 = Q1 - S2
+//   B side: T1 = Q1 - Q0, then T2 = Q3 - T1, T3 = Q3 - Q1, then T4 = T2 - Q2
+template <QuadSums SUMS>
 __global__ void __launch_bounds__(128) quad_pre_kernel(QuadPre q) {
     const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (c >= q.w) return;
     for (long long r = blockIdx.y; r < q.h; r += gridDim.y) {
         const long long o = r * q.ld + c;
-        const float4 Q0 = *reinterpret_cast<const float4*>(q.in[0] + o);
-        const float4 Q1 = *reinterpret_cast<const float4*>(q.in[1] + o);
-        const float4 Q2 = *reinterpret_cast<const float4*>(q.in[2] + o);
-        const float4 Q3 = *reinterpret_cast<const float4*>(q.in[3] + o);
-        float4 X1, X2, X3, X4;
-        if (!SIDE_B) {
-            X1 = add4(Q2, Q3); X2 = sub4(X1, Q0); X3 = sub4(Q0, Q2); X4 = sub4(Q1, X2);
+        auto Q = [&](int i) { return *reinterpret_cast<const float4*>(q.in[i] + o); };
+        auto X = [&](int i) { return *reinterpret_cast<const float4*>(q.out[i - 1] + o); };
+        auto put = [&](int i, float4 v) { *reinterpret_cast<float4*>(q.out[i - 1] + o) = v; };
+        if constexpr (SUMS == kQuadS123) {
+            const float4 Q0 = Q(0), Q2 = Q(2), S1 = add4(Q2, Q(3));
+            put(1, S1);
+            put(2, sub4(S1, Q0));
+            put(3, sub4(Q0, Q2));
+        } else if constexpr (SUMS == kQuadS4) {
+            put(4, sub4(Q(1), X(2)));
+        } else if constexpr (SUMS == kQuadT1) {
+            put(1, sub4(Q(1), Q(0)));
+        } else if constexpr (SUMS == kQuadT23) {
+            const float4 Q3 = Q(3), T1 = X(1), Q1 = Q(1);
+            put(2, sub4(Q3, T1));
+            put(3, sub4(Q3, Q1));
         } else {
-            X1 = sub4(Q1, Q0); X2 = sub4(Q3, X1); X3 = sub4(Q3, Q1); X4 = sub4(X2, Q2);
+            put(4, sub4(X(2), Q(2)));
         }
-        *reinterpret_cast<float4*>(q.out[0] + o) = X1;
-        *reinterpret_cast<float4*>(q.out[1] + o) = X2;
-        *reinterpret_cast<float4*>(q.out[2] + o) = X3;
-        *reinterpret_cast<float4*>(q.out[3] + o) = X4;
     }
 }
 
@@ -1311,11 +1317,16 @@ cudaError_t launch_fp16_scales(const float* A, long long lda, long long M, long 
     return cudaGetLastError();
 }
 
-cudaError_t launch_quad_pre(const QuadPre& q, int side_b, cudaStream_t stream) {
+cudaError_t launch_quad_pre(const QuadPre& q, QuadSums sums, cudaStream_t stream) {
     if (q.h <= 0 || q.w <= 0) return cudaSuccess;
     dim3 grid((unsigned)((q.w + 511) / 512), gy(q.h));
-    if (side_b) quad_pre_kernel<1><<<grid, 128, 0, stream>>>(q);
-    else quad_pre_kernel<0><<<grid, 128, 0, stream>>>(q);
+    switch (sums) {
+        case kQuadS123: quad_pre_kernel<kQuadS123><<<grid, 128, 0, stream>>>(q); break;
+        case kQuadS4: quad_pre_kernel<kQuadS4><<<grid, 128, 0, stream>>>(q); break;
+        case kQuadT1: quad_pre_kernel<kQuadT1><<<grid, 128, 0, stream>>>(q); break;
+        case kQuadT23: quad_pre_kernel<kQuadT23><<<grid, 128, 0, stream>>>(q); break;
+        case kQuadT4: quad_pre_kernel<kQuadT4><<<grid, 128, 0, stream>>>(q); break;
+    }
     return cudaGetLastError();
 }
 
@@ -1498,12 +1509,17 @@ cudaError_t launch_fill(float* p, size_t n, unsigned seed, cudaStream_t stream) 
 // 2-D copy of a rows x cols block between pinned host memory (through its
 // device mapping) and device memory, by SM loads and stores: the host-resident
 // plan's alternative to the copy engines.  float4 when both blocks allow it,
-// four of them in flight per thread, so that a few blocks fill the host link
-// (32 blocks of 512 threads: 211 GB/s in, 193 GB/s out) and the other SMs stay
-// with the compute running beside the copy.
-constexpr int kHostCopyBlocks = 32;
+// four of them in flight per thread; otherwise a warp takes 512 floats of a row
+// at a time, sixteen loads per lane in flight (one load in flight and a division
+// per float: 2216 x 2112 x 6607, odd rows, 1547 us a call; 915 now, panels
+// included).  Few and large blocks: what a copy beside the compute costs is the
+// SMs it touches.  Calls of 8192^3, 3861 x 8164 x 6564, 4000^3 (us) with
+//    8 blocks of 1024 threads: 5250, 2365, 936     64 blocks of 256: 5360, 3055, 1160
+//   12 blocks of 1024:         5177, 2472, 948    152 blocks of 128: 5950, 3157, 1230
+//   16 blocks of 1024:         5190, 2680, 960     32 blocks of 512: 5335, 3113, 1156
+constexpr int kHostCopyBlocks = 12, kHostCopyThreads = 1024;
 constexpr int kHostCopyUnroll = 4;
-__global__ void __launch_bounds__(512) host_copy2d_kernel(const float* __restrict__ src, long long lds,
+__global__ void __launch_bounds__(kHostCopyThreads) host_copy2d_kernel(const float* __restrict__ src, long long lds,
                                                           float* __restrict__ dst, long long ldd, long long rows,
                                                           long long cols, int vec) {
     const long long step = (long long)gridDim.x * blockDim.x;
@@ -1528,10 +1544,20 @@ __global__ void __launch_bounds__(512) host_copy2d_kernel(const float* __restric
             reinterpret_cast<float4*>(dst + r * ldd)[c] = reinterpret_cast<const float4*>(src + r * lds)[c];
         }
     } else {
-        const long long total = rows * cols;
-        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
-            const long long r = i / cols, c = i - r * cols;
-            dst[r * ldd + c] = src[r * lds + c];
+        // a warp takes 512 consecutive floats of a row, sixteen loads per lane in flight
+        const int lane = threadIdx.x & 31;
+        const long long segs = (cols + 511) / 512, total = rows * segs, warps = step >> 5;
+        for (long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < total; i += warps) {
+            const long long r = i / segs, c0 = (i - r * segs) * 512 + lane;
+            const float* s = src + r * lds;
+            float* d = dst + r * ldd;
+            float v[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (c0 + 32 * j < cols) v[j] = s[c0 + 32 * j];
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (c0 + 32 * j < cols) d[c0 + 32 * j] = v[j];
         }
     }
 }
@@ -1541,7 +1567,7 @@ cudaError_t launch_host_copy2d(const float* src, long long lds, float* dst, long
     if (rows <= 0 || cols <= 0) return cudaSuccess;
     const int vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0 &&
                     lds % 4 == 0 && ldd % 4 == 0 && cols % 4 == 0;
-    host_copy2d_kernel<<<kHostCopyBlocks, 512, 0, stream>>>(src, lds, dst, ldd, rows, cols, vec);
+    host_copy2d_kernel<<<kHostCopyBlocks, kHostCopyThreads, 0, stream>>>(src, lds, dst, ldd, rows, cols, vec);
     return cudaGetLastError();
 }
 

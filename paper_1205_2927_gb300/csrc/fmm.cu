@@ -213,7 +213,7 @@ struct fmm_plan_s {
     char* child_ws = nullptr;
     size_t child_ws_bytes = 0;
     cudaStream_t s_h2d = nullptr, s_d2h = nullptr;
-    cudaEvent_t hev[8] = {};
+    cudaEvent_t hev[10] = {};
     // library-default host copies: the input transfers of recent calls that
     // used the copy engines, each bracketed by a pair of timing events in a
     // ring, judged at a later call once complete (callers run ahead of the GPU)
@@ -455,6 +455,7 @@ constexpr bool kFuseLastDefault = true;
 // kHostJudgeBytes, and a plan's first call, are not judged.
 constexpr double kHostStallGBs = 100.0;
 constexpr double kHostJudgeBytes = 64.0 * (1 << 20);
+constexpr int kHostPanels = 8, kPanelTiles = 64;   // panels of a depth-0 product, tiles in one
 
 // Fixed-threshold planner: one more level while every dimension of the next
 // level's leaves stays at or above the cut-off (the recursion point of Sec. 3.1).
@@ -624,9 +625,14 @@ std::vector<std::pair<long long, long long>> rmul_chunks(long long K, int d) {
 // or B transposed for TF32), then one leaf launch per K chunk of the plan's
 // classical recursion: the first writes C = alpha A_0 B_0 + beta C, every later
 // one accumulates C += alpha A_s B_s (Table 1's C = AB, then C += AB leaves).
-// Depth 0 is the single-launch tensor-core GEMM.
+// Depth 0 is the single-launch tensor-core GEMM.  `part`: a panel of the plan's
+// product (its first rows of A and C, or columns of B and C, at the given
+// addresses), with the other operand's planes there from the panel before.
+struct Part { long long M, N; bool a_there, b_there; };
 fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const float* B, float beta, float* C,
-                           cudaStream_t stream) {
+                           cudaStream_t stream, const Part* part = nullptr) {
+    const long long M = part ? part->M : p->M, N = part ? part->N : p->N;
+    const bool do_a = !part || !part->a_there, do_b = !part || !part->b_there;
     const int bf = p->split_kind;
     const long long ld = p->ld16;
     const float* Aop = A;
@@ -638,17 +644,17 @@ fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const flo
         const float* scale = p->mode == kLeafFP16x3P ? p->fp16_scale() : nullptr;
         Stack16 sa{a_raw ? nullptr : p->a16[0], p->a16[1], ld, 0, 1};
         Stack16 sb{p->b16[0], p->b16[1], ld, 0, 1};
-        FMM_CUDA(launch_split16(A, p->lda, p->M, p->K, sa, 0, bf, scale, 0, stream));
-        FMM_CUDA(launch_split16(B, p->ldb, p->K, p->N, sb, 1, bf, scale, 1, stream));
-        p->launches += 2;
+        if (do_a) FMM_CUDA(launch_split16(A, p->lda, M, p->K, sa, 0, bf, scale, 0, stream));
+        if (do_b) FMM_CUDA(launch_split16(B, p->ldb, p->K, N, sb, 1, bf, scale, 1, stream));
+        p->launches += (do_a ? 1 : 0) + (do_b ? 1 : 0);
         p->acct[0] += (double)(p->M * p->K + p->K * p->N) * (4.0 + 2.0 * p->es16()) - (a_raw ? 4.0 * (double)(p->M * p->K) : 0.0);
     } else {
-        FMM_CUDA(launch_transpose(B, p->ldb, p->K, p->N, p->Bt, p->ld_bt, stream));
-        p->launches += 1;
+        if (do_b) FMM_CUDA(launch_transpose(B, p->ldb, p->K, N, p->Bt, p->ld_bt, stream));
+        p->launches += do_b ? 1 : 0;
         p->acct[0] += 8.0 * (double)(p->K * p->N);
         if ((reinterpret_cast<uintptr_t>(A) & 15) || (p->lda % 4)) {
-            FMM_CUDA(launch_copy2d(A, p->lda, p->M, p->K, p->Acopy, p->ld_acopy, stream));
-            p->launches += 1;
+            if (do_a) FMM_CUDA(launch_copy2d(A, p->lda, M, p->K, p->Acopy, p->ld_acopy, stream));
+            p->launches += do_a ? 1 : 0;
             p->acct[0] += 8.0 * (double)(p->M * p->K);
             Aop = p->Acopy;
             lda = p->ld_acopy;
@@ -666,34 +672,34 @@ fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const flo
             const size_t off = (size_t)k0 * p->es16();   // bytes; k0 is a multiple of 8
             for (int i = 0; i < 2; ++i) {
                 if (i == 0 && a_raw) {
-                    if ((s = encode_map16(&args.maps[0], A + k0, bf, kc, p->M, 1, p->lda, p->M * p->lda, kBM,
+                    if ((s = encode_map16(&args.maps[0], A + k0, bf, kc, M, 1, p->lda, M * p->lda, kBM,
                                           p->pair)) != FMM_OK)
                         return s;
                 } else if ((s = encode_map16(&args.maps[i], static_cast<char*>(p->a16[i]) + off, bf,
-                                             i ? p->lo_cols(kc) : kc, p->M, 1, ld, p->M * ld, kBM, p->pair)) != FMM_OK) {
+                                             i ? p->lo_cols(kc) : kc, M, 1, ld, M * ld, kBM, p->pair)) != FMM_OK) {
                     return s;
                 }
                 if ((s = encode_map16(&args.maps[2 + i], static_cast<char*>(p->b16[i]) + off, bf,
-                                      i ? p->lo_cols(kc) : kc, p->N, 1, ld,
-                                      p->N * ld, p->pair ? 128 : p->bn, p->pair)) != FMM_OK)
+                                      i ? p->lo_cols(kc) : kc, N, 1, ld,
+                                      N * ld, p->pair ? 128 : p->bn, p->pair)) != FMM_OK)
                     return s;
             }
             G.map_a = 0; G.map_a_lo = 1; G.map_b = 2; G.map_b_lo = 3;
         } else {
-            if ((s = encode_map(&args.maps[0], Aop + k0, kc, p->M, 1, lda, p->M * lda, kBM)) != FMM_OK) return s;
-            if ((s = encode_map(&args.maps[1], p->Bt + k0, kc, p->N, 1, p->ld_bt, p->N * p->ld_bt,
+            if ((s = encode_map(&args.maps[0], Aop + k0, kc, M, 1, lda, M * lda, kBM)) != FMM_OK) return s;
+            if ((s = encode_map(&args.maps[1], p->Bt + k0, kc, N, 1, p->ld_bt, N * p->ld_bt,
                                 p->pair ? 128 : p->bn)) != FMM_OK)
                 return s;
             G.map_a = 0; G.map_b = 1;
         }
-        G.M = (int)p->M; G.N = (int)p->N; G.K = (int)kc; G.batch = 1;
+        G.M = (int)M; G.N = (int)N; G.K = (int)kc; G.batch = 1;
         G.C = C; G.ldc = p->ldc; G.c_batch_stride = 0;
         G.alpha = alpha; G.beta = first ? beta : 1.0f;
         G.vec_ok = ((reinterpret_cast<uintptr_t>(C) & 15) == 0 && p->ldc % 4 == 0) ? 1 : 0;
         G.corr16 = p->split_kind == kSplitTF32X ? 1 : 0;
         args.num_groups = 1;
         if ((s = run_leaves(p, args, stream)) != FMM_OK) return s;
-        if (!first) p->acct[1] += 8.0 * (double)(p->M * p->N);   // the accumulating launch reads and writes C
+        if (!first) p->acct[1] += 8.0 * (double)(M * N);   // the accumulating launch reads and writes C
         first = false;
     }
     mark(p, 2, stream);
@@ -1501,9 +1507,8 @@ void make_child(const fmm_plan_s* p, fmm_plan_s& c) {
 }
 
 // Host-resident multiply.  The root level runs depth-first over the seven
-// products so that transfers overlap compute: A11, B11 are copied first (P1
-// starts on them), then A12, B21 (P2), then the rest; C11 = P1 + P2 is copied
-// back while P3..P7 run.  Copies run on the plan's two copy streams, ordered
+// products so that transfers overlap compute: each starts once its own quadrants
+// have arrived, and each quadrant of C is copied back while later products run.  Copies run on the plan's two copy streams, ordered
 // after `stream` by events; `stream` waits for the last device-to-host copy.
 fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B, float beta, float* C,
                       cudaStream_t stream) {
@@ -1560,7 +1565,7 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
     FMM_CUDA(cudaStreamWaitEvent(p->s_h2d, ev[0], 0));
     FMM_CUDA(cudaStreamWaitEvent(p->s_d2h, ev[0], 0));
     if (judge) FMM_CUDA(cudaEventRecord(p->hx[slot][0], p->s_h2d));
-    // valid part of quadrant (qi, qj) of an R x W host matrix split at (h, w)
+    // valid part of block (qi, qj) of an R x W host matrix in blocks of h x w
     // host_c / host: the caller's pointer; host_m: its device mapping (SM copies)
     auto copy = [&](bool to_dev, float* dev, long long ldd, const float* host_c, float* host, const void* host_m,
                     long long ldh, long long R, long long W, long long h, long long w, int qi, int qj) -> fmm_status_t {
@@ -1598,34 +1603,72 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
     fmm_status_t s;
 #define FMM_TRY(x) do { if ((s = (x)) != FMM_OK) return s; } while (0)
     if (p->depth == 0) {
-        FMM_TRY(inA(0));
-        FMM_TRY(inB(0));
-        if (beta != 0.0f) FMM_TRY(inC(0));
-        FMM_CUDA(cudaEventRecord(ev[1], p->s_h2d));
+        // Panels of the larger operand and of C, each multiplied as soon as it is there
+        // and copied out while the next ones arrive: kPanelTiles tiles of 256 x 256 at
+        // least, about a wave of the leaf launch.  One panel where the product is one
+        // small launch, and for FP16x3, whose scales need all of A and B.
+        // 3861 x 8164 x 6564 in one panel 3.53 ms, now 2.33 (copy engines; device-resident
+        // 1.34); 3828 x 2664 x 3960 1.01 -> 0.79; 2216 x 2112 x 6607 1.05 -> 0.89.
+        const bool by_rows = p->M >= p->N;
+        const long long side = by_rows ? p->M : p->N, blocks = (side + 255) / 256;
+        const long long tiles = ((p->M + 255) / 256) * ((p->N + 255) / 256);
+        const bool whole = c->small_bn != 0 || c->mode == kLeafFP16x3 || c->mode == kLeafFP16x3P;
+        long long np = whole ? 1 : std::min<long long>(kHostPanels, (tiles + kPanelTiles / 2) / kPanelTiles);
+        if (np < 2) np = whole || blocks < 2 ? 1 : 2;
+        const long long step = (blocks + np - 1) / np * 256;   // rows or columns of a panel
+        FMM_TRY(by_rows ? inB(0) : inA(0));
+        int n = 0;
+        for (long long x = 0; x < side; x += step, ++n) {
+            const long long len = std::min(step, side - x);
+            float* dA = by_rows ? q[0] + x * hk : q[0];
+            float* dB = by_rows ? q[4] : q[4] + x;
+            float* dC = by_rows ? q[23] + x * hn : q[23] + x;
+            const int qi = by_rows ? n : 0, qj = by_rows ? 0 : n;
+            const long long ch = by_rows ? step : hm, cw = by_rows ? hn : step;
+            if (by_rows) FMM_TRY(copy(true, dA, hk, A, nullptr, mapped[0], p->lda, p->M, p->K, step, hk, n, 0));
+            else FMM_TRY(copy(true, dB, hn, B, nullptr, mapped[1], p->ldb, p->K, p->N, hk, step, 0, n));
+            if (beta != 0.0f) FMM_TRY(copy(true, dC, hn, C, nullptr, mapped[2], p->ldc, p->M, p->N, ch, cw, qi, qj));
+            FMM_CUDA(cudaEventRecord(ev[1], p->s_h2d));
+            FMM_CUDA(cudaStreamWaitEvent(stream, ev[1], 0));
+            if (np == 1) {
+                FMM_TRY(execute(c, alpha, dA, dB, beta, dC, stream));
+            } else {
+                const Part part{by_rows ? len : c->M, by_rows ? c->N : len, !by_rows && n > 0, by_rows && n > 0};
+                FMM_TRY(run_classical(c, alpha, dA, dB, beta, dC, stream, &part));
+            }
+            FMM_CUDA(cudaEventRecord(ev[4], stream));
+            FMM_CUDA(cudaStreamWaitEvent(p->s_d2h, ev[4], 0));
+            FMM_TRY(copy(false, dC, hn, nullptr, C, mapped[2], p->ldc, p->M, p->N, ch, cw, qi, qj));
+        }
         if (judge) FMM_CUDA(cudaEventRecord(p->hx[slot][1], p->s_h2d));
-        FMM_CUDA(cudaStreamWaitEvent(stream, ev[1], 0));
-        FMM_TRY(execute(c, alpha, q[0], q[4], beta, q[23], stream));
-        FMM_CUDA(cudaEventRecord(ev[4], stream));
-        FMM_CUDA(cudaStreamWaitEvent(p->s_d2h, ev[4], 0));
-        FMM_TRY(outC(0));
     } else {
-        // Transfers in order of first use, products in an order that lets each
-        // C quadrant leave as soon as its U-chain is complete:
-        //   P1, P2 -> C11;  T sums (all of B) -> P4;  S sums (A21 last) -> P6, P7
-        //   -> C21;  P5 -> C22;  P3 -> C12.
-        // Only the last quadrant's device-to-host copy is not hidden.
-        FMM_TRY(inA(0)); FMM_TRY(inB(0));                        // A11, B11 -> P1
+        // Transfers and products in an order that starts a product as early as any
+        // order can and leaves the fewest after the last input:
+        //   A11 B11 -> P1;  A21 A22 B12 -> P5;  B22 -> P6, P7 -> C22;  A12 -> P3 -> C12;
+        //   B21 -> P4 -> C21;  P2 -> C11.
+        // With a = 1/8 of the input time and c a product's, the last product ends at
+        // max(2a + 7c, 5a + 6c, 6a + 5c, 7a + 3c, 8a + 2c).  Taking A12 and B21 second
+        // (P1 P2 P4 P6 P7 P5 P3) it was max(2a + 7c, 7a + 5c, 8a + 4c): n = 8192, FP32,
+        // copy engines 5.01 -> 4.80 ms.  Only the last quadrant's device-to-host copy is
+        // not hidden.
+        FMM_TRY(inA(0)); FMM_TRY(inB(0));
         FMM_CUDA(cudaEventRecord(ev[1], p->s_h2d));
-        FMM_TRY(inA(1)); FMM_TRY(inB(2));                        // A12, B21 -> P2
+        FMM_TRY(inA(2)); FMM_TRY(inA(3)); FMM_TRY(inB(1));
         FMM_CUDA(cudaEventRecord(ev[2], p->s_h2d));
-        if (beta != 0.0f) FMM_TRY(inC(0));
-        FMM_CUDA(cudaEventRecord(ev[6], p->s_h2d));              // C11 (beta != 0)
-        FMM_TRY(inA(3)); FMM_TRY(inB(1)); FMM_TRY(inB(3));       // A22, B12, B22 -> T sums, P4
+        FMM_TRY(inB(3));
         FMM_CUDA(cudaEventRecord(ev[3], p->s_h2d));
-        FMM_TRY(inA(2));                                         // A21 -> S sums
+        FMM_TRY(inA(1));
         FMM_CUDA(cudaEventRecord(ev[5], p->s_h2d));
-        if (beta != 0.0f) for (int i = 1; i < 4; ++i) FMM_TRY(inC(i));
-        FMM_CUDA(cudaEventRecord(ev[7], p->s_h2d));              // C12, C21, C22 (beta != 0)
+        FMM_TRY(inB(2));
+        FMM_CUDA(cudaEventRecord(ev[6], p->s_h2d));
+        if (beta != 0.0f) {
+            FMM_TRY(inC(3)); FMM_TRY(inC(1));
+            FMM_CUDA(cudaEventRecord(ev[7], p->s_h2d));
+            FMM_TRY(inC(2));
+            FMM_CUDA(cudaEventRecord(ev[8], p->s_h2d));
+            FMM_TRY(inC(0));
+            FMM_CUDA(cudaEventRecord(ev[9], p->s_h2d));
+        }
         if (judge) FMM_CUDA(cudaEventRecord(p->hx[slot][1], p->s_h2d));
         float* P[7];
         for (int i = 0; i < 7; ++i) P[i] = q[16 + i];
@@ -1633,8 +1676,10 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
         for (int i = 0; i < 7; ++i) qp.p[i] = P[i];
         for (int i = 0; i < 4; ++i) qp.c[i] = q[23 + i];
         qp.ld = hn; qp.h = hm; qp.w = hn; qp.alpha = alpha; qp.beta = beta;
-        // C quadrant i is formed on `stream`, then copied out on the d2h stream
-        auto post_out = [&](int i) -> fmm_status_t {
+        // C quadrant i is formed on `stream`, once its old values are there (event e),
+        // then copied out on the d2h stream
+        auto post_out = [&](int i, int e) -> fmm_status_t {
+            if (beta != 0.0f) FMM_CUDA(cudaStreamWaitEvent(stream, ev[e], 0));
             FMM_CUDA(launch_quad_post(qp, i, stream));
             FMM_CUDA(cudaEventRecord(ev[4], stream));
             FMM_CUDA(cudaStreamWaitEvent(p->s_d2h, ev[4], 0));
@@ -1645,23 +1690,28 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
         FMM_CUDA(cudaStreamWaitEvent(stream, ev[1], 0));
         FMM_TRY(execute(c, 1.f, q[0], q[4], 0.f, P[0], stream));   // P1 = A11 B11
         FMM_CUDA(cudaStreamWaitEvent(stream, ev[2], 0));
-        FMM_TRY(execute(c, 1.f, q[1], q[6], 0.f, P[1], stream));   // P2 = A12 B21
-        FMM_CUDA(cudaStreamWaitEvent(stream, ev[6], 0));
-        FMM_TRY(post_out(0));                                      // C11 = alpha U1 + beta C11
+        FMM_CUDA(launch_quad_pre(pa, kQuadS123, stream));
+        FMM_CUDA(launch_quad_pre(pb, kQuadT1, stream));
+        FMM_TRY(execute(c, 1.f, q[8], q[12], 0.f, P[4], stream));  // P5 = S1 T1
         FMM_CUDA(cudaStreamWaitEvent(stream, ev[3], 0));
-        FMM_CUDA(launch_quad_pre(pb, 1, stream));                 // T1..T4
-        FMM_TRY(execute(c, 1.f, q[3], q[15], 0.f, P[3], stream));  // P4 = A22 T4
-        FMM_CUDA(cudaStreamWaitEvent(stream, ev[5], 0));
-        FMM_CUDA(launch_quad_pre(pa, 0, stream));                 // S1..S4
+        FMM_CUDA(launch_quad_pre(pb, kQuadT23, stream));
         FMM_TRY(execute(c, 1.f, q[9], q[13], 0.f, P[5], stream));  // P6 = S2 T2
         FMM_TRY(execute(c, 1.f, q[10], q[14], 0.f, P[6], stream)); // P7 = S3 T3
-        FMM_CUDA(cudaStreamWaitEvent(stream, ev[7], 0));
-        FMM_TRY(post_out(2));                                      // C21 = alpha U6 + beta C21
-        FMM_TRY(execute(c, 1.f, q[8], q[12], 0.f, P[4], stream));  // P5 = S1 T1
-        FMM_TRY(post_out(3));                                      // C22 = alpha U7 + beta C22
+        // C22 = alpha U7 + beta C22; its old values come after all of A and B, so with
+        // beta it waits until P3 has started
+        if (beta == 0.0f) FMM_TRY(post_out(3, 7));
+        FMM_CUDA(cudaStreamWaitEvent(stream, ev[5], 0));
+        FMM_CUDA(launch_quad_pre(pa, kQuadS4, stream));
         FMM_TRY(execute(c, 1.f, q[11], q[7], 0.f, P[2], stream));  // P3 = S4 B22
-        FMM_TRY(post_out(1));                                      // C12 = alpha U5 + beta C12
-        p->launches += 6;
+        if (beta != 0.0f) FMM_TRY(post_out(3, 7));
+        FMM_TRY(post_out(1, 7));                                   // C12 = alpha U5 + beta C12
+        FMM_CUDA(cudaStreamWaitEvent(stream, ev[6], 0));
+        FMM_CUDA(launch_quad_pre(pb, kQuadT4, stream));
+        FMM_TRY(execute(c, 1.f, q[3], q[15], 0.f, P[3], stream));  // P4 = A22 T4
+        FMM_TRY(post_out(2, 8));                                   // C21 = alpha U6 + beta C21
+        FMM_TRY(execute(c, 1.f, q[1], q[6], 0.f, P[1], stream));   // P2 = A12 B21
+        FMM_TRY(post_out(0, 9));                                   // C11 = alpha U1 + beta C11
+        p->launches += 9;
     }
 #undef FMM_TRY
     if (judge && in_bytes >= kHostJudgeBytes) {
@@ -2373,7 +2423,7 @@ fmm_status_t fmm_plan(fmm_plan_t* out, int64_t M, int64_t N, int64_t K, int64_t 
         }
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->s_h2d, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->s_d2h, cudaStreamNonBlocking);
-        for (int i = 0; i < 8 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&p->hev[i], cudaEventDisableTiming);
+        for (int i = 0; i < 10 && e == cudaSuccess; ++i) e = cudaEventCreateWithFlags(&p->hev[i], cudaEventDisableTiming);
         for (int i = 0; i < fmm_plan_s::kJudgeRing * 2 && e == cudaSuccess; ++i)
             e = cudaEventCreate(&p->hx[i / 2][i % 2]);
         if (e != cudaSuccess) { fmm_free(p); return cuda_fail(e, "host-resident plan setup"); }

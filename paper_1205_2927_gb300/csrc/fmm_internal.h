@@ -225,7 +225,10 @@ struct QuadPost {
     long long ld, h, w;
     float alpha, beta;
 };
-cudaError_t launch_quad_pre(const QuadPre& q, int side_b, cudaStream_t stream);
+// Which sums a launch forms: those whose quadrants have arrived (S4 and T2..T4
+// read earlier sums).
+enum QuadSums : int { kQuadS123 = 0, kQuadS4 = 1, kQuadT1 = 2, kQuadT23 = 3, kQuadT4 = 4 };
+cudaError_t launch_quad_pre(const QuadPre& q, QuadSums sums, cudaStream_t stream);
 cudaError_t launch_quad_post(const QuadPost& q, int part, cudaStream_t stream);
 // ------------------------------------------------------------ split hi/lo planes
 // Kinds of split: bf16 (x*s = hi + lo, 16-bit), fp16 (same, 16-bit), tf32
