@@ -259,7 +259,9 @@ fmm_status_t fmm_plan_phase_bytes(fmm_plan_t plan, double* pre_bytes, double* po
 fmm_status_t fmm_wait_selftest(fmm_plan_t plan, int64_t limit_ns, fmm_stream_t stream);
 
 /* Plan inspection: depth, leaf tile width, precision and odd mode the plan
- * uses (after the planner ran); any pointer may be NULL. */
+ * uses (after the planner ran); any pointer may be NULL.  A depth-0 plan whose
+ * leaf tile was left open reports the planner's tile even where it runs as one
+ * small launch, or on pairs of SMs with its last wave of tiles in parts. */
 fmm_status_t fmm_plan_info(fmm_plan_t plan, int* depth, int* leaf_tile, int* precision,
                            int* odd, int* algo);
 

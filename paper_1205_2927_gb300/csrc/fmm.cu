@@ -174,6 +174,7 @@ struct fmm_plan_s {
     int pre16 = 0;
     int split_kind = 0;
     int pair = 0;        // leaves on CTA pairs (cta_group::2), 256 x 256 tiles
+    int parts = 0;       // depth 0, tile left open: the last wave of pair tiles may go out in parts
     int tile_req = 256;  // leaf tile the plan was made for (512: CTA pairs where the precision allows)
     int small_bn = 0;    // depth 0 in one launch of small_gemm.cu: its tile width (0: the leaf path)
     int small_splits = 1;
@@ -468,6 +469,31 @@ int fixed_depth(long long M, long long N, long long K, int cutoff) {
     return d;
 }
 
+// A product of few tiles ends in a wave that most pairs sit out.  Where two or four
+// parts of each of its tiles (128 or 64 columns) fit that wave, they take its place:
+// the same products in the same order, over more pairs.  Returns log2 of the parts.
+// Only where the caller left the tile open: a plan that names its tile (and a candidate
+// that a planner times) runs just that.
+// A part copies all of its A rows, so FP32, bound by copies and operand reads in shared
+// memory, gains less than the 16-bit planes.  Calls at depth 0, us before -> after:
+//   1024 x 1024 x 4096 (16 tiles, 4 parts)  FP32 91 -> 75    BF16x3 69 -> 50    TF32 49.7 -> 47
+//   1300 x 1300 x 5000 (36 tiles, 2 parts)  FP32 121 -> 104  BF16x3 92 -> 71    TF32 63 -> 62
+//   1900 x 3101 x 1503 (76 + 28 tiles, 2)   FP32 86 -> 80    BF16x3 62 -> 56    TF32 67 -> 64
+//   3328 x 3328 x 2048 (152 + 17 tiles, 4)  FP32 152 -> 144  BF16x3 111 -> 102  TF32 80 -> 79
+long long last_wave(long long tiles, long long pairs) { return tiles - (tiles - 1) / pairs * pairs; }
+int tail_parts(long long tiles, long long pairs) {
+    const long long rest = last_wave(tiles, pairs);
+    if (tiles > 4 * pairs) return 0;
+    return 4 * rest <= pairs ? 2 : 2 * rest <= pairs ? 1 : 0;
+}
+// Waves of a depth-0 pair launch, a last one in parts counted by its share of a whole
+// one, fitted over 330 shapes of 256 .. 4095: with these shares the choice below and
+// small_choice's lose 0.3 % to the best of the three kernels on average.
+double pair_waves(long long tiles, fmm_precision_t prec) {
+    const double part = prec == FMM_PREC_FP32 ? 0.7 : prec == FMM_PREC_TF32 ? 0.95 : 0.5;
+    return (double)((tiles + 75) / 76) - (tail_parts(tiles, 76) ? 1.0 - part : 0.0);
+}
+
 // Leaf tile when the caller leaves it open.  Recursive plans: the CTA-pair 256 x 256
 // tile once both output sides of every leaf reach 1024 (from there on it is at
 // least as fast as the single-CTA tile and cuts the per-SM operand traffic by a
@@ -484,6 +510,20 @@ int auto_tile(long long M, long long N, long long K, int depth, const fmm_option
     const long long pair = ((M + 255) / 256) * ((N + 255) / 256), single = ((M + 127) / 128) * ((N + 255) / 256);
     const double rel = fp32 ? (tf32x_leaf(K, 0) ? 0.65 : 0.9) : tf32 ? 0.82 : 1.0;
     return (double)((pair + 75) / 76) * rel <= (double)((single + 151) / 152) ? 512 : 256;
+}
+
+// Whether a depth-0 product whose planner took a single-CTA tile runs on pair tiles all
+// the same, its last wave in parts (tail_parts): the planners' candidates and rules are
+// about whole tiles.  BF16x3 1440 x 913 x 331
+// 24.4 -> 19.9 us, 708 x 1975 x 1904 44.8 -> 34.1; not taken, 45 tiles: 1037 x 2159 x 507
+// 26.8 single, 28.0 pair.
+bool parts_faster(long long M, long long N, long long K, const fmm_options_t& o) {
+    const long long pair = ((M + 255) / 256) * ((N + 255) / 256), single = ((M + 127) / 128) * ((N + 255) / 256);
+    if (std::min(M, N) <= 256 || K <= 0 || !tail_parts(pair, 76)) return false;
+    const double rel = o.precision == FMM_PREC_FP32   ? (tf32x_leaf(K, 0) ? 0.65 : 0.9)
+                       : o.precision == FMM_PREC_TF32 ? 0.82
+                                                      : 1.0;
+    return pair_waves(pair, o.precision) * rel <= (double)((single + 151) / 152);
 }
 
 // Whether a leaf launch takes its tiles in dynamic order: launches over several
@@ -540,8 +580,8 @@ int small_choice(long long M, long long N, long long K, long long lda, fmm_preci
         }
     }
     if (!against_leaf) return best_bn;
-    const double tm = pair ? 256.0 : 128.0, slots = pair ? 76.0 : 152.0;
-    const double waves = std::ceil(std::ceil((double)M / tm) * std::ceil((double)N / 256.0) / slots);
+    const long long tm = pair ? 256 : 128, leaf_tiles = ((M + tm - 1) / tm) * ((N + 255) / 256);
+    const double waves = pair ? pair_waves(leaf_tiles, prec) : (double)((leaf_tiles + 151) / 152);
     const double leaf = m.launches + ((double)M * K * m.a_bytes + (double)K * N * m.b_bytes) / 6e6 +
                         waves * (4.0 + (double)K * (pair ? m.k_pair : m.k));
     // the models miss by up to 15 % on long K, where operands come from DRAM
@@ -585,6 +625,10 @@ fmm_status_t prepare_leaves(fmm_plan_s* p, GemmArgs& args, int mode, bool pair, 
         args.tile_seq = reinterpret_cast<unsigned long long*>(p->tile_sched + 256);
     }
     if (pair) args.fuse_scratch = p->fused ? p->fuse_scratch : nullptr;
+    if (pair && args.tail_shift && !args.tile_counter) {
+        args.tail_tiles = (int)last_wave(t, p->num_sms / 2);
+        args.total_tiles += (long long)args.tail_tiles * ((1 << args.tail_shift) - 1);
+    }
     return FMM_OK;
 }
 
@@ -661,6 +705,7 @@ fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const flo
         }
     }
     mark(p, 1, stream);
+    const int tail = p->pair && p->parts ? tail_parts((M + 255) / 256 * ((N + 255) / 256), p->num_sms / 2) : 0;
     bool first = true;
     for (const auto& [k0, kc] : rmul_chunks(p->K, p->rmul)) {
         if (kc <= 0) continue;
@@ -668,6 +713,8 @@ fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const flo
         memset(&args, 0, sizeof(args));
         fmm_status_t s;
         GemmGroup& G = args.groups[0];
+        args.tail_shift = tail;
+        args.tail_map = 4;
         if (p->pre16) {
             const size_t off = (size_t)k0 * p->es16();   // bytes; k0 is a multiple of 8
             for (int i = 0; i < 2; ++i) {
@@ -685,12 +732,18 @@ fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const flo
                     return s;
             }
             G.map_a = 0; G.map_a_lo = 1; G.map_b = 2; G.map_b_lo = 3;
+            for (int i = 0; tail && i < 2; ++i)
+                if ((s = encode_map16(&args.maps[4 + i], static_cast<char*>(p->b16[i]) + off, bf,
+                                      i ? p->lo_cols(kc) : kc, N, 1, ld, N * ld, 128 >> tail, true)) != FMM_OK)
+                    return s;
         } else {
             if ((s = encode_map(&args.maps[0], Aop + k0, kc, M, 1, lda, M * lda, kBM)) != FMM_OK) return s;
             if ((s = encode_map(&args.maps[1], p->Bt + k0, kc, N, 1, p->ld_bt, N * p->ld_bt,
                                 p->pair ? 128 : p->bn)) != FMM_OK)
                 return s;
             G.map_a = 0; G.map_b = 1;
+            if (tail && (s = encode_map(&args.maps[4], p->Bt + k0, kc, N, 1, p->ld_bt, N * p->ld_bt, 128 >> tail)) != FMM_OK)
+                return s;
         }
         G.M = (int)M; G.N = (int)N; G.K = (int)kc; G.batch = 1;
         G.C = C; G.ldc = p->ldc; G.c_batch_stride = 0;
@@ -1391,8 +1444,10 @@ void make_tmp(fmm_plan_s& t, long long M, long long N, long long K, long long ld
         t.peel_gm = M / gm > 0 ? gm : 0;
         t.peel_gn = N / gn > 0 ? gn : 0;
     }
-    t.bn = bn;
     t.tile_req = bn;
+    t.parts = !t.host && outer == 0 && t.depth == 0 && t.rmul == 0 && o.leaf_tile == 0 ? 1 : 0;
+    if (t.parts && bn != 512 && o.planner != FMM_PLANNER_EXHAUSTIVE && parts_faster(M, N, K, o)) bn = 512;
+    t.bn = bn;
     t.mode = leaf_mode(o.precision);
     t.pre16 = 0;
     t.pair = 0;
@@ -2564,7 +2619,7 @@ fmm_status_t fmm_plan_fuse_last(fmm_plan_t p, int* fused) {
 fmm_status_t fmm_plan_info(fmm_plan_t p, int* depth, int* leaf_tile, int* precision, int* odd, int* algo) {
     if (!p) return FMM_ERR_INVALID_ARG;
     if (depth) *depth = p->rmul ? p->rmul : p->depth;
-    if (leaf_tile) *leaf_tile = (p->pair || (p->host && p->tile_req == 512)) ? 512 : p->bn;
+    if (leaf_tile) *leaf_tile = (p->pair || p->host) ? p->tile_req : p->bn;
     if (precision) *precision = (int)p->opt.precision;
     if (odd) *odd = (int)p->odd;
     if (algo) *algo = (int)p->opt.algo;

@@ -64,7 +64,11 @@ struct GemmArgs {
     const GemmGroup* ext_groups;
     int num_groups;
     int raster_m;                  // tile rows per raster band
-    long long total_tiles;
+    long long total_tiles;         // schedule units: tiles, the last tail_tiles of them in their parts
+    // pair launches in static order: the last tail_tiles tiles go out as 2 or 4 parts
+    // (1 << tail_shift) of 256 rows x 256 >> tail_shift columns, through B maps of the
+    // rows one CTA then stages (hi at tail_map, lo behind it)
+    int tail_tiles, tail_shift, tail_map;
     unsigned* status;              // device status word
     // dynamic tile order of a leaf launch (null: static round robin): the next
     // free tile (zero before the launch), and one ring per CTA (per pair for

@@ -612,8 +612,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
     const int lane = threadIdx.x & 31;
     const CUtensorMap* maps = args.ext_maps ? args.ext_maps : args.maps;
     const GemmGroup* groups = args.ext_groups ? args.ext_groups : args.groups;
-    const int ng = args.num_groups;
-    const long long total = args.total_tiles;   // 256 x 256 pair tiles
+    const long long total = args.total_tiles;   // 256 x 256 pair tiles, then the column parts of the last ones
+    const int tail_shift = args.tail_shift, part_cols = 256 >> tail_shift;
+    const long long whole = total - ((long long)args.tail_tiles << tail_shift);
+    // schedule unit u: its tile and, from `whole` on, which part of it (else -1)
+    auto unit = [&](long long u, int& g, int& b, int& tm, int& tn) -> int {
+        const int part = FUSED || u < whole ? -1 : (int)(u - whole) & ((1 << tail_shift) - 1);
+        decode_tile(groups, args.num_groups, args.raster_m, part < 0 ? u : whole + ((u - whole) >> tail_shift), g, b, tm,
+                    tn);
+        return part;
+    };
     const long long pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     unsigned* status = args.status;
     const bool dyn = args.tile_counter != nullptr;   // dynamic tile order (the pair's ring)
@@ -664,14 +672,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
                 }
                 if (t >= total) break;
                 int g, b, tm, tn;
-                decode_tile(groups, ng, args.raster_m, t, g, b, tm, tn);
+                const int part = unit(t, g, b, tm, tn);
                 const GemmGroup& G = groups[g];
                 const int nk = (G.K + Cfg::kKB - 1) / Cfg::kKB;
                 // the pair's MMA reads B rows [0, ncols / 2) of the tile from CTA 0
                 // and [ncols / 2, ncols) from CTA 1 (ncols < 256 in the last tile
-                // column under the dynamic tile order, as in the MMA issuer)
-                const int ncols = dyn ? (int)tile_cols(G.N, tn, 256) : 256;
-                const int a0 = tm * 256 + (int)rank * Cfg::kRows, b0 = tn * 256 + (int)rank * (ncols / 2);
+                // column under the dynamic tile order, as in the MMA issuer; a
+                // part's B boxes have just its rows)
+                const int ncols = part >= 0 ? part_cols : dyn ? (int)tile_cols(G.N, tn, 256) : 256;
+                const int a0 = tm * 256 + (int)rank * Cfg::kRows;
+                const int b0 = tn * 256 + (part > 0 ? part * part_cols : 0) + (int)rank * (ncols / 2);
+                const CUtensorMap* map_b = maps + (part >= 0 ? args.tail_map : G.map_b);
+                const CUtensorMap* map_b_lo = maps + (part >= 0 ? args.tail_map + 1 : G.map_b_lo);
+                const uint32_t tx =
+                    2 * (Cfg::kStageBytes - (part >= 0 ? (Cfg::kPlain ? 1 : 2) * (Cfg::kRows - part_cols / 2) * 128 : 0));
                 for (int pp = 0; pp < kProducts && ok; ++pp) {
                 const int leaf = FUSED ? b * 7 + kFusedOrder[pp] : b;
                 const int ab = leaf + G.a_batch_off, bb = leaf + G.b_batch_off;
@@ -682,18 +696,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
                     // CTA 0 arms its full barrier with the bytes of both CTAs; a
                     // peer copy that lands first only drives the tx-count below
                     // zero, which the arming arrival brings back
-                    if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), 2 * Cfg::kStageBytes);
+                    if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), tx);
                     const uint32_t ah = stage0 + stage * Cfg::kStageBytes;
                     const int x = kb * Cfg::kKB;
                     if constexpr (Cfg::kPlain) {
                         tma_load_3d_pair(ah, maps + G.map_a, full_bar(stage), x, a0, ab);
-                        tma_load_3d_pair(ah + Cfg::kRows * 128, maps + G.map_b, full_bar(stage), x, b0, bb);
+                        tma_load_3d_pair(ah + Cfg::kRows * 128, map_b, full_bar(stage), x, b0, bb);
                     } else {
                         const uint32_t bh = ah + Cfg::kRows * 128, al = bh + Cfg::kRows * 128, bl = al + Cfg::kRows * 128;
                         tma_load_3d_pair(ah, maps + G.map_a, full_bar(stage), x, a0, ab);
-                        tma_load_3d_pair(bh, maps + G.map_b, full_bar(stage), x, b0, bb);
+                        tma_load_3d_pair(bh, map_b, full_bar(stage), x, b0, bb);
                         tma_load_3d_pair(al, maps + G.map_a_lo, full_bar(stage), x, a0, ab);
-                        tma_load_3d_pair(bl, maps + G.map_b_lo, full_bar(stage), x, b0, bb);
+                        tma_load_3d_pair(bl, map_b_lo, full_bar(stage), x, b0, bb);
                     }
                     ++issued;
                     if (++stage == Cfg::kStages) { stage = 0; phase ^= 1u; }
@@ -721,9 +735,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
                                         : pair + (long long)i * npairs;
                 if (t < 0 || t >= total) break;
                 int g, b, tm, tn;
-                decode_tile(groups, ng, args.raster_m, t, g, b, tm, tn);
+                const int part = unit(t, g, b, tm, tn);
                 const int nk = (groups[g].K + Cfg::kKB - 1) / Cfg::kKB;
-                const uint32_t ncols = dyn ? tile_cols(groups[g].N, tn, 256) : 256u;
+                const uint32_t ncols = part >= 0 ? (uint32_t)part_cols : dyn ? tile_cols(groups[g].N, tn, 256) : 256u;
                 const uint32_t idesc = idesc_with_n(idesc_full, ncols);
                 const uint32_t idesc_corr = idesc_with_n(idesc_corr_full, ncols);
                 const bool corr16 = MODE == kLeaf3xTF32P && groups[g].corr16 != 0;
@@ -815,7 +829,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
             }
             if (t < 0 || t >= total) break;
             int g, b, tm, tn;
-            decode_tile(groups, ng, args.raster_m, t, g, b, tm, tn);
+            const int part = unit(t, g, b, tm, tn);
             const GemmGroup& G = groups[g];
             const int row0 = tm * 256 + (int)rank * Cfg::kRows + q * 32;
             const int rows = min(32, G.M - row0);   // <= 0: this warp's rows are padding
@@ -829,11 +843,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
             if constexpr (!FUSED) {
             float* crow = G.C + (long long)b * G.c_batch_stride + (long long)row0 * G.ldc;
 #pragma unroll 1
-            for (int c = 0; c < 256 / 32; ++c) {
+            for (int c = 0; c < (part >= 0 ? part_cols : 256) / 32; ++c) {
                 uint32_t r[32];
                 tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * 256 + c * 32), r);
                 tmem_ld_wait();
-                const int col0 = tn * 256 + c * 32;
+                const int col0 = tn * 256 + (part > 0 ? part * part_cols : 0) + c * 32;
                 if (rows > 0 && col0 < G.N) {
                     float v[32];
 #pragma unroll
@@ -942,6 +956,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
 // gain (3500 x 3500 x 1000: FP32 91.7 -> 92.5, TF32 55.4 -> 56.7).
 static long long even_grid(const GemmArgs& args, long long cap) {
     if (args.total_tiles <= cap) return args.total_tiles;
+    if (args.tail_tiles) return cap;   // the parts fill the last wave
     const long long waves = (args.total_tiles + cap - 1) / cap;
     if (waves > 4 || args.ext_groups || args.num_groups != 1 || args.groups[0].K < 1024) return cap;
     return (args.total_tiles + waves - 1) / waves;
