@@ -547,8 +547,9 @@ bool dynamic_order(const fmm_plan_s* p, const GemmArgs& args) {
 //   small  7 + waves * (2 + steps of 32 columns / splits * c), c the step of a
 //          128 x {32, 64, 128} tile
 //   leaf   launches, operand passes at 6 TB/s, waves * (4 + K * k)
-// (FP32 512^3 10.5 us against 31, 573 x 452 x 2103 25 against 74, 1024^3 21
-// against 37; not taken: 1500^3 45 against 48, 900 x 4000 x 1000 62 against 50).
+// (FP32, against the leaf path in whole tiles: 512^3 10.5 us against 31, 573 x 452 x
+// 2103 25 against 74, 1024^3 21 against 37, 28 in parts; not taken: 900 x 4000 x 1000 62
+// against 50).
 // Splitting K shortens the accumulators' chains; it is limited to chains whose
 // results then move by less than 2e-5 (FP32: 1.9e-8 per instruction, three per 8
 // columns).  Returns the tile width, or 0 for the leaf path.

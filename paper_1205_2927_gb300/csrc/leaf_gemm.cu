@@ -535,6 +535,11 @@ __global__ void __launch_bounds__(LeafCfg<BN, MODE>::kThreads, 1) leaf_gemm_kern
 // 8192 depth 2 2.39 -> 1.88 ms.  Six half stages of 32 KB, or alternating which
 // kind goes first, changed nothing beyond 3 %.
 //
+// The last tail_tiles tiles of a depth-0 launch can go out as 2 or 4 column parts
+// (GemmArgs::tail_shift): units of 256 x 128 or 256 x 64 whose B boxes hold 64 or 32
+// rows per CTA, so a part copies its A rows and its own B rows only.  A part takes
+// 0.7 of a tile's time in FP32 and 0.5 to 0.6 with 16-bit planes.
+//
 // FUSED: the last Winograd level inside the leaf launch.  A schedule unit is one
 // 256 x 256 tile position of one last-level node; the pair computes the node's
 // seven products at that position back to back, in the order P1, P2, P6, P7,
