@@ -123,7 +123,7 @@ typedef struct {
                                   tiles in M and N, off otherwise and at depth 4) */
     int host_copy;             /* host-resident plans: how A, B, C cross the host link.
                                   1: copy engines (cudaMemcpy2DAsync); 2: SM loads and stores
-                                  on the device mapping of the pinned memory (32 blocks; the
+                                  on the device mapping of the pinned memory (a few blocks; the
                                   same link rate one way, no duplex, but no stall where the
                                   copy engines stall; copy engines for memory without a device
                                   mapping); 0: library default: copy engines until a call's

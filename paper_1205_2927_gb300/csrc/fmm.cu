@@ -1562,6 +1562,47 @@ void make_child(const fmm_plan_s* p, fmm_plan_s& c) {
     }
 }
 
+// Schedules of a host-resident root: quadrants in (0..3 = 11, 12, 21, 22), sums and
+// products as soon as the quadrants before their kArrive are there, quadrants of C
+// out as soon as their products are.  With beta, C's old quadrants come in too.
+enum HostOp : unsigned char { kInA, kInB, kInC, kArrive, kSums, kProduct, kOut, kHostEnd };
+enum HostWhen : unsigned char { kAlways, kIfBeta, kIfNoBeta };
+struct HostStep {
+    HostOp op;
+    unsigned char arg;   // quadrant; event; QuadSums; product 1..7
+    HostWhen when = kAlways;
+};
+const HostStep kOrderFast[] = {   // P1 P5 P6 P7 P3 P4 P2
+    {kInA, 0}, {kInB, 0}, {kArrive, 1}, {kProduct, 1},
+    {kInA, 2}, {kInA, 3}, {kInB, 1}, {kArrive, 2}, {kSums, kQuadS123}, {kSums, kQuadT1}, {kProduct, 5},
+    {kInB, 3}, {kArrive, 3}, {kSums, kQuadT23}, {kProduct, 6}, {kProduct, 7}, {kOut, 3, kIfNoBeta},
+    {kInA, 1}, {kArrive, 4}, {kSums, kQuadS4}, {kProduct, 3}, {kOut, 1, kIfNoBeta},
+    {kInB, 2}, {kArrive, 5}, {kSums, kQuadT4},
+    {kInC, 3, kIfBeta}, {kInC, 1, kIfBeta}, {kArrive, 6, kIfBeta}, {kOut, 3, kIfBeta}, {kOut, 1, kIfBeta},
+    {kProduct, 4}, {kInC, 2, kIfBeta}, {kArrive, 7, kIfBeta}, {kOut, 2},
+    {kProduct, 2}, {kInC, 0, kIfBeta}, {kArrive, 8, kIfBeta}, {kOut, 0}, {kHostEnd, 0}};
+const HostStep kOrderSlow[] = {   // P1 P2 P4 P6 P7 P5 P3
+    {kInA, 0}, {kInB, 0}, {kArrive, 1}, {kProduct, 1},
+    {kInA, 1}, {kInB, 2}, {kArrive, 2}, {kProduct, 2}, {kInC, 0, kIfBeta}, {kArrive, 3, kIfBeta}, {kOut, 0},
+    {kInA, 3}, {kInB, 1}, {kInB, 3}, {kArrive, 4}, {kSums, kQuadT1}, {kSums, kQuadT23}, {kSums, kQuadT4}, {kProduct, 4},
+    {kInA, 2}, {kArrive, 5}, {kSums, kQuadS123}, {kSums, kQuadS4}, {kProduct, 6}, {kProduct, 7},
+    {kInC, 1, kIfBeta}, {kInC, 2, kIfBeta}, {kInC, 3, kIfBeta}, {kArrive, 6, kIfBeta}, {kOut, 2},
+    {kProduct, 5}, {kOut, 3}, {kProduct, 3}, {kOut, 1}, {kHostEnd, 0}};
+
+// With a = 1/8 of the input time and c a product's, the last product ends at
+// max(2a + 7c, 5a + 6c, 6a + 5c, 7a + 3c, 8a + 2c) in the first order and at
+// max(2a + 7c, 7a + 5c, 8a + 4c) in the second: the first is ahead while c < 2a.  The
+// copies beside it slow a product by about a tenth, so the line lies at 1.8, c by
+// the rates of products of 4096 and 8192 (FP32 400 TFLOP/s), a at 205 GB/s.  First
+// and second order, ms a call (copy engines; SM copies): n = 8192 4.80, 5.02; 5.16,
+// 5.29; n = 12000 11.71, 12.00; 12.37, 12.44; n = 16384 27.7, 27.0; 30.6, 29.5.
+const HostStep* host_order(const fmm_plan_s* p) {
+    const double rate = p->opt.precision == FMM_PREC_FP32 ? 400e12 : p->opt.precision == FMM_PREC_TF32 ? 900e12 : 600e12;
+    const double c = 2.0 * (double)p->hm * (double)p->hn * (double)p->hk / rate;
+    const double a = ((double)p->M * p->K + (double)p->K * p->N) * 4.0 / 8.0 / 205e9;
+    return c < 1.8 * a ? kOrderFast : kOrderSlow;
+}
+
 // Host-resident multiply.  The root level runs depth-first over the seven
 // products so that transfers overlap compute: each starts once its own quadrants
 // have arrived, and each quadrant of C is copied back while later products run.  Copies run on the plan's two copy streams, ordered
@@ -1613,6 +1654,7 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
                        p->hx_bytes[slot] <= 0.0;
     p->host_calls += 1;
     double in_bytes = 0.0;
+    const HostStep* const order = p->depth > 0 ? host_order(p) : nullptr;
     fmm_plan_s* c = p->child;
     cudaEvent_t* ev = p->hev;
     float** q = p->hq;
@@ -1631,8 +1673,8 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
         if (to_dev) in_bytes += 4.0 * (double)(rows * cols);
         if (sm_copy) {
             float* hm_ = const_cast<float*>(static_cast<const float*>(host_m)) + r0 * ldh + c0;
-            if (to_dev) FMM_CUDA(launch_host_copy2d(hm_, ldh, dev, ldd, rows, cols, p->s_h2d));
-            else FMM_CUDA(launch_host_copy2d(dev, ldd, hm_, ldh, rows, cols, p->s_d2h));
+            if (to_dev) FMM_CUDA(launch_host_copy2d(hm_, ldh, dev, ldd, rows, cols, order == kOrderSlow, p->s_h2d));
+            else FMM_CUDA(launch_host_copy2d(dev, ldd, hm_, ldh, rows, cols, order == kOrderSlow, p->s_d2h));
             p->launches += 1;
             return FMM_OK;
         }
@@ -1698,75 +1740,42 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
         }
         if (judge) FMM_CUDA(cudaEventRecord(p->hx[slot][1], p->s_h2d));
     } else {
-        // Transfers and products in an order that starts a product as early as any
-        // order can and leaves the fewest after the last input:
-        //   A11 B11 -> P1;  A21 A22 B12 -> P5;  B22 -> P6, P7 -> C22;  A12 -> P3 -> C12;
-        //   B21 -> P4 -> C21;  P2 -> C11.
-        // With a = 1/8 of the input time and c a product's, the last product ends at
-        // max(2a + 7c, 5a + 6c, 6a + 5c, 7a + 3c, 8a + 2c).  Taking A12 and B21 second
-        // (P1 P2 P4 P6 P7 P5 P3) it was max(2a + 7c, 7a + 5c, 8a + 4c): n = 8192, FP32,
-        // copy engines 5.01 -> 4.80 ms.  Only the last quadrant's device-to-host copy is
-        // not hidden.
-        FMM_TRY(inA(0)); FMM_TRY(inB(0));
-        FMM_CUDA(cudaEventRecord(ev[1], p->s_h2d));
-        FMM_TRY(inA(2)); FMM_TRY(inA(3)); FMM_TRY(inB(1));
-        FMM_CUDA(cudaEventRecord(ev[2], p->s_h2d));
-        FMM_TRY(inB(3));
-        FMM_CUDA(cudaEventRecord(ev[3], p->s_h2d));
-        FMM_TRY(inA(1));
-        FMM_CUDA(cudaEventRecord(ev[5], p->s_h2d));
-        FMM_TRY(inB(2));
-        FMM_CUDA(cudaEventRecord(ev[6], p->s_h2d));
-        if (beta != 0.0f) {
-            FMM_TRY(inC(3)); FMM_TRY(inC(1));
-            FMM_CUDA(cudaEventRecord(ev[7], p->s_h2d));
-            FMM_TRY(inC(2));
-            FMM_CUDA(cudaEventRecord(ev[8], p->s_h2d));
-            FMM_TRY(inC(0));
-            FMM_CUDA(cudaEventRecord(ev[9], p->s_h2d));
-        }
-        if (judge) FMM_CUDA(cudaEventRecord(p->hx[slot][1], p->s_h2d));
         float* P[7];
         for (int i = 0; i < 7; ++i) P[i] = q[16 + i];
         QuadPost qp{};
         for (int i = 0; i < 7; ++i) qp.p[i] = P[i];
         for (int i = 0; i < 4; ++i) qp.c[i] = q[23 + i];
         qp.ld = hn; qp.h = hm; qp.w = hn; qp.alpha = alpha; qp.beta = beta;
-        // C quadrant i is formed on `stream`, once its old values are there (event e),
-        // then copied out on the d2h stream
-        auto post_out = [&](int i, int e) -> fmm_status_t {
-            if (beta != 0.0f) FMM_CUDA(cudaStreamWaitEvent(stream, ev[e], 0));
-            FMM_CUDA(launch_quad_post(qp, i, stream));
-            FMM_CUDA(cudaEventRecord(ev[4], stream));
-            FMM_CUDA(cudaStreamWaitEvent(p->s_d2h, ev[4], 0));
-            return outC(i);
-        };
-        QuadPre pa{{q[0], q[1], q[2], q[3]}, {q[8], q[9], q[10], q[11]}, hk, hm, hk};
-        QuadPre pb{{q[4], q[5], q[6], q[7]}, {q[12], q[13], q[14], q[15]}, hn, hk, hn};
-        FMM_CUDA(cudaStreamWaitEvent(stream, ev[1], 0));
-        FMM_TRY(execute(c, 1.f, q[0], q[4], 0.f, P[0], stream));   // P1 = A11 B11
-        FMM_CUDA(cudaStreamWaitEvent(stream, ev[2], 0));
-        FMM_CUDA(launch_quad_pre(pa, kQuadS123, stream));
-        FMM_CUDA(launch_quad_pre(pb, kQuadT1, stream));
-        FMM_TRY(execute(c, 1.f, q[8], q[12], 0.f, P[4], stream));  // P5 = S1 T1
-        FMM_CUDA(cudaStreamWaitEvent(stream, ev[3], 0));
-        FMM_CUDA(launch_quad_pre(pb, kQuadT23, stream));
-        FMM_TRY(execute(c, 1.f, q[9], q[13], 0.f, P[5], stream));  // P6 = S2 T2
-        FMM_TRY(execute(c, 1.f, q[10], q[14], 0.f, P[6], stream)); // P7 = S3 T3
-        // C22 = alpha U7 + beta C22; its old values come after all of A and B, so with
-        // beta it waits until P3 has started
-        if (beta == 0.0f) FMM_TRY(post_out(3, 7));
-        FMM_CUDA(cudaStreamWaitEvent(stream, ev[5], 0));
-        FMM_CUDA(launch_quad_pre(pa, kQuadS4, stream));
-        FMM_TRY(execute(c, 1.f, q[11], q[7], 0.f, P[2], stream));  // P3 = S4 B22
-        if (beta != 0.0f) FMM_TRY(post_out(3, 7));
-        FMM_TRY(post_out(1, 7));                                   // C12 = alpha U5 + beta C12
-        FMM_CUDA(cudaStreamWaitEvent(stream, ev[6], 0));
-        FMM_CUDA(launch_quad_pre(pb, kQuadT4, stream));
-        FMM_TRY(execute(c, 1.f, q[3], q[15], 0.f, P[3], stream));  // P4 = A22 T4
-        FMM_TRY(post_out(2, 8));                                   // C21 = alpha U6 + beta C21
-        FMM_TRY(execute(c, 1.f, q[1], q[6], 0.f, P[1], stream));   // P2 = A12 B21
-        FMM_TRY(post_out(0, 9));                                   // C11 = alpha U1 + beta C11
+        const QuadPre pa{{q[0], q[1], q[2], q[3]}, {q[8], q[9], q[10], q[11]}, hk, hm, hk};
+        const QuadPre pb{{q[4], q[5], q[6], q[7]}, {q[12], q[13], q[14], q[15]}, hn, hk, hn};
+        // operands of P1..P7 among the buffers: A quadrants 0-3, B 4-7, S 8-11, T 12-15
+        static const int operand[7][2] = {{0, 4}, {1, 6}, {11, 7}, {3, 15}, {8, 12}, {9, 13}, {10, 14}};
+        // every copy in is queued before the first product
+        for (const HostStep* t = order; t->op != kHostEnd; ++t) {
+            if ((t->when == kIfBeta && beta == 0.0f) || (t->when == kIfNoBeta && beta != 0.0f)) continue;
+            if (t->op == kInA) FMM_TRY(inA(t->arg));
+            else if (t->op == kInB) FMM_TRY(inB(t->arg));
+            else if (t->op == kInC) FMM_TRY(inC(t->arg));
+            else if (t->op == kArrive) FMM_CUDA(cudaEventRecord(ev[t->arg], p->s_h2d));
+        }
+        if (judge) FMM_CUDA(cudaEventRecord(p->hx[slot][1], p->s_h2d));
+        for (const HostStep* t = order; t->op != kHostEnd; ++t) {
+            if ((t->when == kIfBeta && beta == 0.0f) || (t->when == kIfNoBeta && beta != 0.0f)) continue;
+            if (t->op == kArrive) {
+                FMM_CUDA(cudaStreamWaitEvent(stream, ev[t->arg], 0));
+            } else if (t->op == kSums) {
+                const QuadSums x = (QuadSums)t->arg;
+                FMM_CUDA(launch_quad_pre(x == kQuadS123 || x == kQuadS4 ? pa : pb, x, stream));
+            } else if (t->op == kProduct) {
+                const int i = t->arg - 1;
+                FMM_TRY(execute(c, 1.f, q[operand[i][0]], q[operand[i][1]], 0.f, P[i], stream));
+            } else if (t->op == kOut) {   // formed on `stream`, then copied out on the d2h stream
+                FMM_CUDA(launch_quad_post(qp, t->arg, stream));
+                FMM_CUDA(cudaEventRecord(ev[0], stream));
+                FMM_CUDA(cudaStreamWaitEvent(p->s_d2h, ev[0], 0));
+                FMM_TRY(outC(t->arg));
+            }
+        }
         p->launches += 9;
     }
 #undef FMM_TRY

@@ -48,3 +48,20 @@ def test_panels_equal_device_plan(F, m, n, k, prec, how, beta):
     assert d.device_status() == 0
     d.close()
     assert np.array_equal(hC.numpy(), dC[:, :n].cpu().numpy())
+
+
+@pytest.mark.parametrize("m,n", [(1500, 1300), (14200, 14100)])   # each order of the root's products
+@pytest.mark.parametrize("beta", [0.0, -0.5])
+def test_root_orders_exact(F, m, n, beta):
+    import torch
+    k = 72
+    A, B, C0 = I.small_int((m, k), 91, r=2), I.small_int((k, n), 92, r=2), I.small_int((m, n), 93, r=4)
+    hA, hB, hC = (torch.from_numpy(x).pin_memory() for x in (A, B, C0))
+    p = F.Plan(m, n, k, depth=1, host_operands=1, host_copy="engine")
+    p(hA, hB, hC, alpha=2.0, beta=beta)
+    torch.cuda.synchronize()
+    assert p.device_status() == 0
+    p.close()
+    ref = 2.0 * (torch.from_numpy(A).cuda().double() @ torch.from_numpy(B).cuda().double())
+    ref += beta * torch.from_numpy(C0).cuda().double()
+    assert torch.equal(hC.cuda(), ref.float())
