@@ -130,7 +130,7 @@ __device__ __forceinline__ float sum8(float x) {   // over the eight sample grou
 // which updates the parameters itself (batches whose workspace holds no two rows).
 // Blocks take tiles blockIdx.x * per, ... (per tiles each).
 template <bool ALONE>
-__global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* __restrict__ X, const float* __restrict__ T,
+__global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* X, const float* T,
                                                           int per, float* __restrict__ rows, AdamArgs a) {
     extern __shared__ float4 train_smem[];
     TrainSmem& S = *reinterpret_cast<TrainSmem*>(train_smem);
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* __restric
 // Second kernel: 32 parameters per block, 16 warps over the rows (warp w adds
 // rows w, w + 16, ...), then the 16 sums in order, then Adam (bias-corrected) in
 // place.
-__global__ void __launch_bounds__(512) mlp_adam_kernel(const float* __restrict__ rows, int nrows, AdamArgs a) {
+__global__ void __launch_bounds__(512) mlp_adam_kernel(const float* rows, int nrows, AdamArgs a) {
     __shared__ float part[16][32];
     dep_start();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;

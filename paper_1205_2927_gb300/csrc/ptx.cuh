@@ -26,7 +26,8 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // Kernels launched by launch_dep.  dep_wait: until the kernel before this one has
-// completed and its writes are visible.  dep_trigger: once every block has called it
+// completed and its writes are visible (to plain loads; no __ldg and no const
+// __restrict__ in such a kernel).  dep_trigger: once every block has called it
 // (or ended), the next such kernel's blocks may become resident.
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

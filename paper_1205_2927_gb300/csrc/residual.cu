@@ -24,9 +24,9 @@ namespace {
 // go one at a time.  Warp sums, then the 8 warp sums in a fixed order.  One
 // row per block keeps the grid many waves deep (16384 rows: 13.5 waves).
 template <typename Acc, typename Vec, typename Out>
-__global__ void __launch_bounds__(256) rowdot_kernel(const float* __restrict__ X, long long ld, long long rows,
-                                                     long long cols, const Vec* __restrict__ v,
-                                                     Out* __restrict__ out, const double* __restrict__ sub,
+__global__ void __launch_bounds__(256) rowdot_kernel(const float* X, long long ld, long long rows,
+                                                     long long cols, const Vec* v,
+                                                     Out* __restrict__ out, const double* sub,
                                                      int vec4) {
     __shared__ Acc warp_sum[8];
     dep_start();
@@ -40,14 +40,14 @@ __global__ void __launch_bounds__(256) rowdot_kernel(const float* __restrict__ X
         const float4* x4 = reinterpret_cast<const float4*>(xr);
 #pragma unroll 4
         for (long long g = t; g < groups; g += 256) {
-            const float4 xv = __ldg(x4 + g);
+            const float4 xv = x4[g];
             Acc v0, v1, v2, v3;
             if constexpr (std::is_same<Vec, float>::value) {
-                const float4 q = __ldg(reinterpret_cast<const float4*>(v) + g);
+                const float4 q = reinterpret_cast<const float4*>(v)[g];
                 v0 = q.x; v1 = q.y; v2 = q.z; v3 = q.w;
             } else {
-                const double2 q0 = __ldg(reinterpret_cast<const double2*>(v) + 2 * g);
-                const double2 q1 = __ldg(reinterpret_cast<const double2*>(v) + 2 * g + 1);
+                const double2 q0 = reinterpret_cast<const double2*>(v)[2 * g];
+                const double2 q1 = reinterpret_cast<const double2*>(v)[2 * g + 1];
                 v0 = (Acc)q0.x; v1 = (Acc)q0.y; v2 = (Acc)q1.x; v3 = (Acc)q1.y;
             }
             a0 += (Acc)xv.x * v0;
@@ -108,11 +108,11 @@ __device__ __forceinline__ void widen(const float (&x)[N], double (&d)[N]) {
 // 16-byte rows (four sums a row), 8 on others (one sum a row; two rows took
 // 1.6 times as long as four); below 304 blocks of that, one row per block.
 template <typename Vec, int R, bool VEC4>
-__global__ void __launch_bounds__(256, 3) rowdot64_kernel(const float* __restrict__ X, long long ld,
+__global__ void __launch_bounds__(256, 3) rowdot64_kernel(const float* X, long long ld,
                                                                      long long rows, long long cols,
-                                                                     const Vec* __restrict__ v,
+                                                                     const Vec* v,
                                                                      double* __restrict__ out,
-                                                                     const double* __restrict__ sub) {
+                                                                     const double* sub) {
     __shared__ double warp_sum[8][R];
     dep_start();
     const long long row0 = (long long)blockIdx.x * R;
@@ -128,15 +128,15 @@ __global__ void __launch_bounds__(256, 3) rowdot64_kernel(const float* __restric
         for (long long g = t; g < groups; g += 256) {
             float4 q[R];
 #pragma unroll
-            for (int r = 0; r < R; ++r) q[r] = __ldg(reinterpret_cast<const float4*>(xr[r]) + g);
+            for (int r = 0; r < R; ++r) q[r] = reinterpret_cast<const float4*>(xr[r])[g];
             double w[4];
             if constexpr (std::is_same<Vec, float>::value) {
-                const float4 f = __ldg(reinterpret_cast<const float4*>(v) + g);
+                const float4 f = reinterpret_cast<const float4*>(v)[g];
                 const float ff[4] = {f.x, f.y, f.z, f.w};
                 widen(ff, w);
             } else {
-                const double2 d0 = __ldg(reinterpret_cast<const double2*>(v) + 2 * g);
-                const double2 d1 = __ldg(reinterpret_cast<const double2*>(v) + 2 * g + 1);
+                const double2 d0 = reinterpret_cast<const double2*>(v)[2 * g];
+                const double2 d1 = reinterpret_cast<const double2*>(v)[2 * g + 1];
                 w[0] = d0.x; w[1] = d0.y; w[2] = d1.x; w[3] = d1.y;
             }
 #pragma unroll
@@ -154,13 +154,13 @@ __global__ void __launch_bounds__(256, 3) rowdot64_kernel(const float* __restric
     for (long long c = c0 + t; c < cols; c += 256) {
         float q[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) q[r] = __ldg(xr[r] + c);
+        for (int r = 0; r < R; ++r) q[r] = xr[r][c];
         double d[R], w[1];
         if constexpr (std::is_same<Vec, float>::value) {
-            const float f[1] = {__ldg(v + c)};
+            const float f[1] = {v[c]};
             widen(f, w);
         } else {
-            w[0] = __ldg(v + c);
+            w[0] = v[c];
         }
         widen(q, d);
 #pragma unroll

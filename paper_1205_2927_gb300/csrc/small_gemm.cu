@@ -180,12 +180,12 @@ __global__ void __launch_bounds__(544, 1) small_gemm_kernel(const SmallArgs args
                 if (whole && args.a_vec) {
 #pragma unroll
                     for (int j = 0; j < G; j += 4) {
-                        const float4 v = __ldg(reinterpret_cast<const float4*>(p + j));
+                        const float4 v = *reinterpret_cast<const float4*>(p + j);
                         a[buf][i][j] = v.x; a[buf][i][j + 1] = v.y; a[buf][i][j + 2] = v.z; a[buf][i][j + 3] = v.w;
                     }
                 } else {
 #pragma unroll
-                    for (int j = 0; j < G; ++j) a[buf][i][j] = whole || ac * G + j < left ? __ldg(p + j) : 0.0f;
+                    for (int j = 0; j < G; ++j) a[buf][i][j] = whole || ac * G + j < left ? p[j] : 0.0f;
                 }
             }
             if (has_b) {
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(544, 1) small_gemm_kernel(const SmallArgs args
                     const float* p = pb[i] + bo;
                     const int k = (t + NL * i) / BN * G;
 #pragma unroll
-                    for (int j = 0; j < G; ++j, p += args.ldb) b[buf][i][j] = whole || k + j < left ? __ldg(p) : 0.0f;
+                    for (int j = 0; j < G; ++j, p += args.ldb) b[buf][i][j] = whole || k + j < left ? *p : 0.0f;
                 }
             }
         };
