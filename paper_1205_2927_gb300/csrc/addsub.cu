@@ -515,7 +515,8 @@ __global__ void __launch_bounds__(128) quad_post_kernel(QuadPost q) {
 // the leaf launch only after far more data than L2 holds has passed, and they
 // must not push out the operand lines a fused pass reads again.
 //   tf32x:       hi = rn_tf32(x) (trunc_tf32(x) where the leaves read the raw operand), and in the
-//                other plane bf16(hi) and bf16(x - hi), 32 columns of each per 128-byte line
+//                other plane bf16(hi) and bf16(x - hi), 32 columns of each per 128-byte line (zeros for an
+//                infinity, which the hi plane alone carries)
 // Two values to bf16, nearest even, saturating at the largest finite value.
 __device__ __forceinline__ uint32_t bf16x2_sat(float x0, float x1) {
     uint32_t r;
@@ -535,10 +536,15 @@ __device__ __forceinline__ void split_store(void* hi_plane, void* lo_plane, long
         } else {
             h = f4(tf32_trunc(v.x), tf32_trunc(v.y), tf32_trunc(v.z), tf32_trunc(v.w));
         }
+        // an infinity's product is its hi's alone: x - hi would be NaN
+        float4 l = sub4(v, h);
+        if (isinf(v.x)) h.x = l.x = 0.f;
+        if (isinf(v.y)) h.y = l.y = 0.f;
+        if (isinf(v.z)) h.z = l.z = 0.f;
+        if (isinf(v.w)) h.w = l.w = 0.f;
         uint16_t* hl = static_cast<uint16_t*>(lo_plane) + tf32x_off(o);
         __stcs(reinterpret_cast<uint2*>(hl), make_uint2(bf16x2_sat(h.x, h.y), bf16x2_sat(h.z, h.w)));
-        __stcs(reinterpret_cast<uint2*>(hl + 32),
-               make_uint2(bf16x2_sat(v.x - h.x, v.y - h.y), bf16x2_sat(v.z - h.z, v.w - h.w)));
+        __stcs(reinterpret_cast<uint2*>(hl + 32), make_uint2(bf16x2_sat(l.x, l.y), bf16x2_sat(l.z, l.w)));
         return;
     }
     if constexpr (KIND == kSplitTF32) {
