@@ -514,9 +514,8 @@ __global__ void __launch_bounds__(128) quad_post_kernel(QuadPost q) {
 // The planes are written with evict-first (streaming) stores: they are read by
 // the leaf launch only after far more data than L2 holds has passed, and they
 // must not push out the operand lines a fused pass reads again.
-//   tf32x:       hi = rn_tf32(x) (trunc_tf32(x) where the leaves read the raw operand), and in the
-//                other plane bf16(hi) and bf16(x - hi), 32 columns of each per 128-byte line (zeros for an
-//                infinity, which the hi plane alone carries)
+//   tf32x:       hi = rn_tf32(x), and in the other plane bf16(hi) and bf16(x - hi), 32 columns of
+//                each per 128-byte line (zeros for an infinity, which the hi plane alone carries)
 // Two values to bf16, nearest even, saturating at the largest finite value.
 __device__ __forceinline__ uint32_t bf16x2_sat(float x0, float x1) {
     uint32_t r;
@@ -526,16 +525,15 @@ __device__ __forceinline__ uint32_t bf16x2_sat(float x0, float x1) {
 // 16-bit offset of hi (lo: + 32) of the element at offset o of a tf32x correction plane.
 __device__ __forceinline__ long long tf32x_off(long long o) { return 2 * (o & ~31LL) + (o & 31); }
 
-template <int KIND>
+// RAW (A of a depth-0 product): hi = x as for tf32, whether the leaves read the operand
+// itself (no hi plane) or its copy, so that a product has the same bits at any alignment
+// of A; tf32x corrections are then those of trunc_tf32(x).
+template <int KIND, bool RAW = false>
 __device__ __forceinline__ void split_store(void* hi_plane, void* lo_plane, long long o, float4 v, float sc) {
     if constexpr (KIND == kSplitTF32X) {
-        float4 h;
-        if (hi_plane) {
-            h = f4(tf32_round_hi(v.x), tf32_round_hi(v.y), tf32_round_hi(v.z), tf32_round_hi(v.w));
-            __stcs(reinterpret_cast<float4*>(static_cast<float*>(hi_plane) + o), h);
-        } else {
-            h = f4(tf32_trunc(v.x), tf32_trunc(v.y), tf32_trunc(v.z), tf32_trunc(v.w));
-        }
+        float4 h = RAW ? f4(tf32_trunc(v.x), tf32_trunc(v.y), tf32_trunc(v.z), tf32_trunc(v.w))
+                       : f4(tf32_round_hi(v.x), tf32_round_hi(v.y), tf32_round_hi(v.z), tf32_round_hi(v.w));
+        if (hi_plane) __stcs(reinterpret_cast<float4*>(static_cast<float*>(hi_plane) + o), RAW ? v : h);
         // an infinity's product is its hi's alone: x - hi would be NaN
         float4 l = sub4(v, h);
         if (isinf(v.x)) h.x = l.x = 0.f;
@@ -624,7 +622,7 @@ __global__ void __launch_bounds__(256) split16_kernel(const float* X, long long 
             const int g = tid + 256 * j;
             const long long r = r0 + (g >> 5), c = c0 + 4 * (g & 31);
             // ld is a multiple of 8, so a group of 4 never crosses a row: padding columns get zeros
-            if (r < rows && c < plane_cols<KIND>(cols)) split_store<KIND>(out.hi, out.lo, r * out.ld + c, v[j], sc);
+            if (r < rows && c < plane_cols<KIND>(cols)) split_store<KIND, true>(out.hi, out.lo, r * out.ld + c, v[j], sc);
         }
         return;
     }
@@ -1194,7 +1192,7 @@ __global__ void __launch_bounds__(256) batched_split_kernel(const SplitJob* __re
             if (KIND == kSplitTF32X && !J.corr16) {
                 if (r < J.rows && c < J.cols) split_store<kSplitTF32>(J.dst, J.lo, r * J.ldd + c, v[j], sc);
             } else if (r < J.rows && c < plane_cols<KIND>(J.cols)) {
-                split_store<KIND>(J.dst, J.lo, r * J.ldd + c, v[j], sc);
+                split_store<KIND, true>(J.dst, J.lo, r * J.ldd + c, v[j], sc);
             }
         }
         return;

@@ -242,11 +242,12 @@ cudaError_t launch_quad_post(const QuadPost& q, int part, cudaStream_t stream);
 // Kinds of split: bf16 (x*s = hi + lo, 16-bit), fp16 (same, 16-bit), tf32
 // (fp32 planes: hi = x itself -- the tensor core reads trunc_tf32(x) -- and
 // lo = rn_tf32(x - trunc_tf32(x))).
-// tf32x (CTA-pair leaves): hi = the nearest TF32 value of x as fp32 (or the raw
-// operand itself, read truncated), and in place of the lo plane one of the same
-// size whose 128-byte lines hold, per 32 columns, 32 bf16 values of hi and then
-// 32 of x - hi: the operands of the two correction products.  Its columns from
-// the matrix's last to the next multiple of 32 are written as zeros.
+// tf32x (CTA-pair leaves): hi = the nearest TF32 value of x as fp32 (A at depth 0:
+// x itself, read truncated, in place where its rows are aligned), and in place of
+// the lo plane one of the same size whose 128-byte lines hold, per 32 columns, 32
+// bf16 values of hi and then 32 of x - hi: the operands of the two correction
+// products.  Its columns from the matrix's last to the next multiple of 32 are
+// written as zeros.
 enum SplitKind : int { kSplitBF16 = 0, kSplitFP16 = 1, kSplitTF32 = 2, kSplitTF32X = 3 };
 inline bool split_is32(int kind) { return kind == kSplitTF32 || kind == kSplitTF32X; }
 // A stack of split matrices: child c of node p at plane + (p * nchild + c) *
