@@ -61,8 +61,18 @@ typedef enum {
 typedef enum {
     FMM_PREC_FP32 = 0,   /* hi*hi + hi*lo + lo*hi of TF32 hi parts, fp32 accumulate (FP32-class):
                             three TF32 products, or, on CTA-pair leaves of a range of lengths
-                            at depths 0 to 2 where its total error is the smaller, one TF32
-                            product and the two corrections in bf16 */
+                            at depths 0 to 2, one TF32 product and the two corrections in bf16.
+                            The second form adds less often to the accumulator, which truncates:
+                            dense operands come out closer to float64 (1.9e-5 against 2.9e-5 in
+                            the 2-norm at depth 0, K = 4096).  Its single terms are rougher:
+                            within 2^-17 of |a b|, an element of A (of B) times a power of two
+                            within 2^-19 (2^-20); with three TF32 products 2^-19, 2^-22.  So
+                            where few terms meet, permutations, diagonals or a few non-zeros
+                            per column, it is the less exact: A times a permutation 6e-7 rms
+                            and 1.9e-6 at worst (8e-8, 2.4e-7), A times a diagonal 1.1e-6 and
+                            7.5e-6 (2.3e-7, 1.4e-6), integers pass unchanged below 2^19 in A
+                            and 2^20 in B (2^22).  Callers who need three TF32 products for
+                            such operands set leaf_tile to 128 or 256. */
     FMM_PREC_TF32 = 1,   /* one TF32 product, fp32 accumulate */
     FMM_PREC_BF16X3 = 2, /* bfloat16 hi/lo split, 3 products, fp32 accumulate */
     FMM_PREC_FP16X3 = 3  /* IEEE half hi/lo split with power-of-two scaling, 3 products */

@@ -426,13 +426,18 @@ long long leaf_k(long long K, int d, bool peel) {
 
 // Whether FP32 leaves of k columns at this depth, on CTA pairs, take the TF32
 // product with bf16 corrections (kSplitTF32X) instead of three TF32 products.
-// Their operands carry about 2^-20.7 of rounding (three TF32 products: 2^-23),
-// but the truncating accumulator, 1.9e-8 per instruction and leaf, gets two
-// instructions per 16 columns of K fewer.  From the lower limits on the sum of
-// both is no larger than with three TF32 products (depth 0: equal near K = 150;
-// a level amplifies the operands' part by 2.6, the accumulator's hardly).  Up to
-// the upper limits the two results agree within 2e-5 in the 2-norm (depth 0,
-// K = 4096: 1.0e-5; depth 2, K = 2048: 1.03e-5; depth 3, K = 2048: 2.4e-5, not taken).
+// A term's rounding is larger (rms 1.1e-6 against 2.3e-7), but the truncating
+// accumulator, 1.9e-8 per instruction and leaf, gets two instructions per 16 columns
+// of K fewer.  From the lower limits on the error of dense operands, both parts of it,
+// is no larger than with three TF32 products (2-norm against float64, depth 0: equal
+// near K = 150, K = 192 1.38e-6 and 1.55e-6, K = 4096 1.93e-5 and 2.91e-5; depth 1,
+// K = 4096 9.97e-6 and 1.50e-5; depth 2, K = 8192 1.23e-5 and 1.69e-5; a level amplifies
+// the terms' part by 2.6, the accumulator's hardly).  Neither K nor the depth tells a
+// sparse operand, whose terms' rounding shows: fmm.h says what it comes to, and a named
+// single-CTA tile keeps the three products.  The upper limits are where the two results
+// part by more than 2e-5 in the 2-norm (depth 0, K = 4096: 1.0e-5; depth 2, K = 2048:
+// 1.03e-5; depth 3, K = 2048: 2.4e-5, not taken): beyond them the change of form would
+// move results that callers have compared.
 bool tf32x_leaf(long long k, int depth) {
     switch (depth) {
         case 0: return k >= 192 && k <= 6144;
