@@ -366,15 +366,16 @@ fmm_status_t fmm_set_cost_model(const float* params, const float* mean6, const f
  * Computes C <- alpha * A * B + beta * C (row-major device pointers, the same
  * conventions as fmm_gemm) in one launch over FP32 (3xTF32) tensor-core tiles
  * whose CTAs split and turn the operands themselves and share long K ranges, so
- * it needs no temporaries.  M, N and K must each be <= 1024; larger sizes return
+ * it needs no temporaries; where C shares memory with A or B, that operand is
+ * copied first, into an array of the library (8 MB).  M, N and K must each be <= 1024; larger sizes return
  * FMM_ERR_INVALID_ARG with the limit in fmm_last_error().  The call allocates
  * nothing (no cudaMalloc/cudaFree, no host heap, no allocating library
  * routine).  The first call on a device looks up the device address of the
- * library's status word (once per device, with that device current); make that
+ * library's status word and array (once per device, with that device current); make that
  * first call before any stream capture.  Every call clears the status word, so
  * fmm_gemm_static_status reports on the last call; calls that overlap on the GPU
  * (different streams, or different threads on the same device) share that one
- * word. */
+ * word, and the array of copies. */
 fmm_status_t fmm_gemm_static(int64_t M, int64_t N, int64_t K, float alpha, const float* A, int64_t lda,
                              const float* B, int64_t ldb, float beta, float* C, int64_t ldc,
                              fmm_stream_t stream);

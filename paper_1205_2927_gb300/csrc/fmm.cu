@@ -594,6 +594,19 @@ int small_choice(long long M, long long N, long long K, long long lda, fmm_preci
     return best < (K <= 4096 ? 0.97 : 0.85) * leaf ? best_bn : 0;
 }
 
+// Whether an operand (rows x cols) and C (M x N) share an element.  Column blocks of
+// one buffer, rows equally long, do not; other address ranges that meet count as shared.
+bool shares(const float* X, long long ldx, long long rows, long long cols, const float* C, long long ldc, long long M,
+            long long N) {
+    if (rows <= 0 || cols <= 0 || M <= 0 || N <= 0) return false;
+    const uintptr_t x0 = reinterpret_cast<uintptr_t>(X), x1 = x0 + 4 * (uintptr_t)((rows - 1) * ldx + cols);
+    const uintptr_t c0 = reinterpret_cast<uintptr_t>(C), c1 = c0 + 4 * (uintptr_t)((M - 1) * ldc + N);
+    if (x1 <= c0 || c1 <= x0) return false;
+    if (ldx != ldc || (x0 - c0) % 4) return true;
+    const long long off = ((long long)(c0 - x0) / 4 % ldx + ldx) % ldx;   // C's first column in X's rows
+    return off < cols || off + N > ldx;
+}
+
 SmallArgs small_args(long long M, long long N, long long K, float alpha, const float* A, long long lda, const float* B,
                      long long ldb, float beta, float* C, long long ldc, unsigned* status) {
     SmallArgs a;
@@ -688,8 +701,10 @@ fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const flo
     const float* Aop = A;
     long long lda = p->lda;
     // FP32 (3xTF32): the hi plane is the raw value, so an aligned A is read in
-    // place and only its lo plane is written
-    const bool a_raw = p->pre16 && split_is32(bf) && (reinterpret_cast<uintptr_t>(A) & 15) == 0 && p->lda % 4 == 0;
+    // place and only its lo plane is written; not where the leaves store C over it
+    const bool a_ok = (reinterpret_cast<uintptr_t>(A) & 15) == 0 && p->lda % 4 == 0 &&
+                      !shares(A, p->lda, M, p->K, C, p->ldc, M, N);
+    const bool a_raw = p->pre16 && split_is32(bf) && a_ok;
     if (p->pre16) {
         const float* scale = p->mode == kLeafFP16x3P ? p->fp16_scale() : nullptr;
         Stack16 sa{a_raw ? nullptr : p->a16[0], p->a16[1], ld, 0, 1};
@@ -702,7 +717,7 @@ fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const flo
         if (do_b) FMM_CUDA(launch_transpose(B, p->ldb, p->K, N, p->Bt, p->ld_bt, stream));
         p->launches += do_b ? 1 : 0;
         p->acct[0] += 8.0 * (double)(p->K * p->N);
-        if ((reinterpret_cast<uintptr_t>(A) & 15) || (p->lda % 4)) {
+        if (!a_ok) {
             if (do_a) FMM_CUDA(launch_copy2d(A, p->lda, M, p->K, p->Acopy, p->ld_acopy, stream));
             p->launches += do_a ? 1 : 0;
             p->acct[0] += 8.0 * (double)(p->M * p->K);
@@ -1083,7 +1098,10 @@ fmm_status_t execute(fmm_plan_s* p, float alpha, const float* A, const float* B,
         p->launches += 2;
         p->acct[0] += 4.0 * (double)(p->M * p->K + p->K * p->N);
     }
-    if (p->small_bn) {
+    // the small kernel stores C while its other blocks still read A and B; a C that
+    // shares memory with them goes by the leaf path, whose passes copy them first
+    if (p->small_bn && !shares(A, p->lda, p->M, p->K, C, p->ldc, p->M, p->N) &&
+        !shares(B, p->ldb, p->K, p->N, C, p->ldc, p->M, p->N)) {
         SmallArgs a = small_args(p->M, p->N, p->K, alpha, A, p->lda, B, p->ldb, beta, C, p->ldc, p->status);
         if (p->opt.precision == FMM_PREC_FP16X3) a.scale = p->fp16_scale();
         const int mode = p->opt.precision == FMM_PREC_TF32     ? kSmallTF32
@@ -1715,7 +1733,11 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
         const bool by_rows = p->M >= p->N;
         const long long side = by_rows ? p->M : p->N, blocks = (side + 255) / 256;
         const long long tiles = ((p->M + 255) / 256) * ((p->N + 255) / 256);
-        const bool whole = c->small_bn != 0 || c->mode == kLeafFP16x3 || c->mode == kLeafFP16x3P;
+        // One panel, too, where C shares memory with A or B: all of them is in before any
+        // of C goes out.
+        const bool whole = c->small_bn != 0 || c->mode == kLeafFP16x3 || c->mode == kLeafFP16x3P ||
+                           shares(A, p->lda, p->M, p->K, C, p->ldc, p->M, p->N) ||
+                           shares(B, p->ldb, p->K, p->N, C, p->ldc, p->M, p->N);
         long long np = whole ? 1 : std::min<long long>(kHostPanels, (tiles + kPanelTiles / 2) / kPanelTiles);
         if (np < 2) np = whole || blocks < 2 ? 1 : 2;
         const long long step = (blocks + np - 1) / np * 256;   // rows or columns of a panel
@@ -2645,29 +2667,34 @@ fmm_status_t fmm_plan_info(fmm_plan_t p, int* depth, int* leaf_tile, int* precis
 
 // ------------------------------------------------------------------------------------------
 // Allocation-free entry point: one launch of the small-product kernel, which needs
-// no temporaries; only its status word lives in device memory compiled into the
-// library.  Calls that overlap on the GPU share that word.
+// no temporaries; its status word, and room for copies of operands that C shares
+// memory with, lie in device memory compiled into the library.  Calls that overlap
+// on the GPU share both.
 namespace {
 constexpr long long kStaticMaxDim = 1024;
-__device__ __align__(256) unsigned g_static_status[64];
-// device address of the word, per device; filled on a device's first call and
+struct StaticArea {
+    unsigned status[64];
+    float copies[2][kStaticMaxDim * kStaticMaxDim];   // of A and of B
+};
+__device__ __align__(256) unsigned char g_static_area[sizeof(StaticArea)];
+// device address of the area, per device; filled on a device's first call and
 // read under g_mu, so host threads making first calls at once do not race
-unsigned* g_static_status_addr[64] = {};
+StaticArea* g_static_area_addr[64] = {};
 
-// The word's device address on the current device (looked up once per device,
+// The area's device address on the current device (looked up once per device,
 // with that device current: the host-side name of the array is not a device
 // address).
-fmm_status_t static_status(unsigned** out) {
+fmm_status_t static_area(StaticArea** out) {
     int dev = 0;
     FMM_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return FMM_ERR_NO_DEVICE;
     std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_static_status_addr[dev]) {
+    if (!g_static_area_addr[dev]) {
         void* ptr = nullptr;
-        FMM_CUDA(cudaGetSymbolAddress(&ptr, g_static_status));
-        g_static_status_addr[dev] = static_cast<unsigned*>(ptr);
+        FMM_CUDA(cudaGetSymbolAddress(&ptr, g_static_area));
+        g_static_area_addr[dev] = static_cast<StaticArea*>(ptr);
     }
-    *out = g_static_status_addr[dev];
+    *out = g_static_area_addr[dev];
     return FMM_OK;
 }
 }  // namespace
@@ -2688,8 +2715,9 @@ extern "C" fmm_status_t fmm_gemm_static(int64_t M, int64_t N, int64_t K, float a
     DeviceInfo di;
     fmm_status_t s = device_info(&di);
     if (s != FMM_OK) return s;
-    unsigned* status = nullptr;
-    if ((s = static_status(&status)) != FMM_OK) return s;
+    StaticArea* area = nullptr;
+    if ((s = static_area(&area)) != FMM_OK) return s;
+    unsigned* status = area->status;
     if (alpha == 0.0f || K == 0) {
         // no kernel of this call can report into the status word: clear it so
         // that fmm_gemm_static_status describes this call
@@ -2698,6 +2726,20 @@ extern "C" fmm_status_t fmm_gemm_static(int64_t M, int64_t N, int64_t K, float a
         return FMM_OK;
     }
     if (!A || !B) return FMM_ERR_INVALID_ARG;
+    // the kernel stores C while its other blocks still read A and B: an operand that
+    // shares memory with C is read from a copy
+    if (shares(A, lda, M, K, C, ldc, M, N)) {
+        const long long ld = rup(K, 4);
+        FMM_CUDA(launch_copy2d(A, lda, M, K, area->copies[0], ld, stream));
+        A = area->copies[0];
+        lda = ld;
+    }
+    if (shares(B, ldb, K, N, C, ldc, M, N)) {
+        const long long ld = rup(N, 4);
+        FMM_CUDA(launch_copy2d(B, ldb, K, N, area->copies[1], ld, stream));
+        B = area->copies[1];
+        ldb = ld;
+    }
     // K shared by at least two CTAs beyond one step: its accumulator chains are then
     // no longer than those of one Winograd level's leaves
     SmallArgs a = small_args(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, status);
@@ -2712,8 +2754,9 @@ extern "C" fmm_status_t fmm_gemm_static_status(fmm_stream_t stream) {
     DeviceInfo di;
     fmm_status_t s = device_info(&di);
     if (s != FMM_OK) return s;
-    unsigned* status = nullptr;
-    if ((s = static_status(&status)) != FMM_OK) return s;
+    StaticArea* area = nullptr;
+    if ((s = static_area(&area)) != FMM_OK) return s;
+    unsigned* status = area->status;
     FMM_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
     unsigned w = 0;
     FMM_CUDA(cudaMemcpy(&w, status, sizeof(w), cudaMemcpyDeviceToHost));
