@@ -310,7 +310,11 @@ fmm_status_t fmm_residual(int64_t M, int64_t N, int64_t K, const float* A, int64
  *
  * fmm_autotune times every candidate on the caller's device buffers A, B, C
  * (C is overwritten) with CUDA events on `stream` (1 warm-up + reps timed
- * runs, median) and synchronises.  depths/tiles/times_ms receive up to 16
+ * runs, median) and synchronises.  Each candidate is timed with its leaf tile
+ * named, whole tiles of the leaf kernels; so are the times that a cost model
+ * learns from.  FMM_PLANNER_EXHAUSTIVE times each as the plan made from it
+ * runs: a depth-0 plan that leaves its tile open may be one small launch, or
+ * have its last wave in parts.  depths/tiles/times_ms receive up to 16
  * entries, *count their number; any may be NULL.  workspace: at least
  * *workspace_needed bytes (the largest candidate); with workspace == NULL
  * only *workspace_needed is set. */

@@ -1856,10 +1856,14 @@ fmm_status_t choose_mlp(long long M, long long N, long long K, const fmm_options
     return FMM_OK;
 }
 
-// Time each candidate on A, B, C (dense row-major) with the workspace `ws`.
+// Time each candidate on A, B, C (dense row-major) with the workspace `ws`.  as_plan:
+// each as the plan that is made from it runs, at depth 0 as one small launch or with its
+// last wave in parts where make_tmp says so (a plan chosen by the tiles' own times
+// could pick a level against a depth 0 that it would not run: 768^3 FP32 at depth 1, 22
+// us, beside 11 at depth 0); else leaf tiles as themselves, a table of depths and tiles.
 fmm_status_t autotune_core(long long M, long long N, long long K, const fmm_options_t& o, const float* A,
                            const float* B, float* C, char* ws, size_t ws_bytes, const Cand* c, int n, int reps,
-                           float* times, cudaStream_t stream) {
+                           bool as_plan, float* times, cudaStream_t stream) {
     DeviceInfo di;
     fmm_status_t s;
     if ((s = device_info(&di)) != FMM_OK) return s;
@@ -1871,7 +1875,7 @@ fmm_status_t autotune_core(long long M, long long N, long long K, const fmm_opti
         fmm_plan_s t;
         fmm_options_t od = o;
         od.host_operands = 0;   // candidates are timed on device operands
-        od.leaf_tile = c[i].bn;   // leaf tiles as themselves (make_tmp's small products have none)
+        if (!as_plan) od.leaf_tile = c[i].bn;
         make_tmp(t, M, N, K, K, N, N, od, c[i].depth, c[i].bn);
         size_t need = 0;
         layout(&t, nullptr, &need);
@@ -1954,7 +1958,7 @@ fmm_status_t plan_choose(long long M, long long N, long long K, long long lda, l
     FMM_CUDA(launch_fill(sA, (size_t)M * K, 12345u, stream));
     FMM_CUDA(launch_fill(sB, (size_t)K * N, 54321u, stream));
     float times[16];
-    fmm_status_t s = autotune_core(M, N, K, o, sA, sB, sC, base, align_up(mx, 256), c, n, 1, times, stream);
+    fmm_status_t s = autotune_core(M, N, K, o, sA, sB, sC, base, align_up(mx, 256), c, n, 1, true, times, stream);
     if (s != FMM_OK) return s;
     int b = 0;
     for (int i = 1; i < n; ++i)
@@ -2016,8 +2020,8 @@ fmm_status_t fmm_autotune(int64_t M, int64_t N, int64_t K, const fmm_options_t* 
     if (workspace_bytes < mx) return FMM_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(workspace) & 255) return FMM_ERR_ALIGNMENT;
     float t[16];
-    s = autotune_core(M, N, K, o, A, B, C, static_cast<char*>(workspace), workspace_bytes, c, n, reps, t,
-                      (cudaStream_t)stream);
+    s = autotune_core(M, N, K, o, A, B, C, static_cast<char*>(workspace), workspace_bytes, c, n, reps, false,
+                      t, (cudaStream_t)stream);
     if (s != FMM_OK) return s;
     if (times_ms)
         for (int i = 0; i < n; ++i) times_ms[i] = t[i];
