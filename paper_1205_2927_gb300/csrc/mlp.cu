@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(NT, 3) mlp_train_kernel(const float* X, const 
                 const float d = on ? dy * S.w3[ug + 16 * u] : 0.f;
                 S.dz2[row][ug + 16 * u] = d;
                 gb2[u] += d;
-                gw3[u] += on ? dy * z[q][u] : 0.f;
+                gw3[u] += dy * (z[q][u] > 0.f ? z[q][u] : 0.f);   // dy = 0 beyond the batch; a dy of NaN shows
             }
         }
         __syncthreads();
