@@ -552,9 +552,10 @@ bool dynamic_order(const fmm_plan_s* p, const GemmArgs& args) {
 //   small  7 + waves * (2 + steps of 32 columns / splits * c), c the step of a
 //          128 x {32, 64, 128} tile
 //   leaf   launches, operand passes at 6 TB/s, waves * (4 + K * k)
-// (FP32, against the leaf path in whole tiles: 512^3 10.5 us against 31, 573 x 452 x
-// 2103 25 against 74, 1024^3 21 against 37, 28 in parts; not taken: 900 x 4000 x 1000 62
-// against 50).
+// (FP32, against the leaf path in whole pair tiles: 768^3 11 us against 30, 573 x 452 x
+// 2103 22 against 55, 1024^3 18 against 35, 28 in parts, 512^3 15.5 against 21: `resident`
+// has 16 clusters of 8, and the GPUs measured since hold 15; not taken: 900 x 4000 x 1000,
+// 37.4 by the leaf path).
 // Splitting K shortens the accumulators' chains; it is limited to chains whose
 // results then move by less than 2e-5 (FP32: 1.9e-8 per instruction, three per 8
 // columns).  Returns the tile width, or 0 for the leaf path.
@@ -1491,8 +1492,9 @@ void make_tmp(fmm_plan_s& t, long long M, long long N, long long K, long long ld
     }
     // depth 0, by whichever planner, with the leaf tile left open: small products in
     // one launch where the models favour it.  A caller who fixes depth 0 for leaves of
-    // 1024 and more keeps the leaf path, whose operand passes fmm_plan_phase_bytes
-    // reports
+    // 1024 and more keeps the leaf path (1024^3: 28 us, 18 in one launch): such plans
+    // promise its operand passes (fmm_plan_phase_bytes) and, in whole tiles or parts, the
+    // bits of the plan that names the tile
     t.small_bn = 0;
     if (!t.host && outer == 0 && t.depth == 0 && t.rmul == 0 && o.leaf_tile == 0 && M > 0 && N > 0 && K > 0 &&
         (std::min(M, N) < 1024 || o.depth < 0))

@@ -14,8 +14,8 @@
 // shared-memory pipe sets (operand loads, split stores and MMA reads; 512 loader
 // threads keep loads two steps ahead, 256 took 1.0 us a step): 0.60 / 0.65 / 0.80
 // us per 32 columns of K at tiles of 32 / 64 / 128 columns in FP32.  Calls:
-// 700 x 515 x 901 45.7 us by the leaf path, 16.4 this way; 512^3 30.9 and 10.5;
-// 573 x 452 x 2103 74 and 25.
+// 700 x 515 x 901 38 us by the leaf path, 13.7 this way; 768^3 30 and 11; 573 x
+// 452 x 2103 55 and 22; 512^3 21 and 15.5 (16 clusters of 8, of which 15 fit at once).
 //
 //   warps 0..15 loaders: coalesced global reads (rows of A 128 bytes at a time,
 //               B by columns), split, 16-byte swizzled shared-memory stores; after
