@@ -48,8 +48,8 @@ __device__ __forceinline__ void store4(float* p, float4 v, bool vec, long long n
 
 // grid: x over column groups of 4, y over rows (strided), z over nodes.
 template <bool VEC, int SIDE_B, bool FULL>
-__global__ void __launch_bounds__(128) pre_add_kernel(View P, long long h, long long w, Stack out) {
-    dep_start();
+__global__ void __launch_bounds__(128) pre_add_kernel(View P, long long h, long long w, Stack out, int dep) {
+    if (dep) dep_start();
     const long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (c >= w) return;
     const long long node = blockIdx.z;
@@ -875,7 +875,6 @@ __device__ __forceinline__ void split_store1(void* hi_plane, void* lo_plane, lon
 template <int SIDE_B, int KIND>
 __global__ void __launch_bounds__(256, 2) pre_add3_kernel(View P, long long h, long long w, Stack16 out,
                                                        const float* scale) {
-    dep_start();
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= w) return;
     const float sc = scale ? scale[SIDE_B] : 1.0f;
@@ -1240,13 +1239,20 @@ cudaError_t launch_pre_add(const View& parent, long long nodes, const Stack& out
     const bool vec = aligned16(parent.ptr) && aligned16(out.ptr) && parent.ld % 4 == 0 && w % 4 == 0 &&
                      parent.node_stride % 4 == 0 && out.ld % 4 == 0 && out.child_stride % 4 == 0;
     dim3 grid((unsigned)((w + 4 * 128 - 1) / (4 * 128)), gy(h), (unsigned)nodes);
-#define FMM_PRE(V, S, F) launch_dep(pre_add_kernel<V, S, F>, grid, 128, 0, stream, parent, h, w, out)
+    // dependent on the pass before it while a row keeps two warps busy; blocks of less work
+    // pay more for the wait than it hides (5700 x 4441 x 312, TF32, depth 3, rows of 160, 80
+    // and 40: pre-additions 74 us in plain order, 102 dependent; n = 1500, depth 2, rows of
+    // 752 and 376: 31 and 26)
+    const int dep = w >= 256;
+#define FMM_PRE(V, S, F)                                                                              \
+    if (dep) launch_dep(pre_add_kernel<V, S, F>, grid, 128, 0, stream, parent, h, w, out, 1);           \
+    else pre_add_kernel<V, S, F><<<grid, 128, 0, stream>>>(parent, h, w, out, 0)
     if (vec) {
-        if (side_b) { if (full) FMM_PRE(true, 1, true); else FMM_PRE(true, 1, false); }
-        else        { if (full) FMM_PRE(true, 0, true); else FMM_PRE(true, 0, false); }
+        if (side_b) { if (full) { FMM_PRE(true, 1, true); } else { FMM_PRE(true, 1, false); } }
+        else        { if (full) { FMM_PRE(true, 0, true); } else { FMM_PRE(true, 0, false); } }
     } else {
-        if (side_b) { if (full) FMM_PRE(false, 1, true); else FMM_PRE(false, 1, false); }
-        else        { if (full) FMM_PRE(false, 0, true); else FMM_PRE(false, 0, false); }
+        if (side_b) { if (full) { FMM_PRE(false, 1, true); } else { FMM_PRE(false, 1, false); } }
+        else        { if (full) { FMM_PRE(false, 0, true); } else { FMM_PRE(false, 0, false); } }
     }
 #undef FMM_PRE
     return cudaGetLastError();
@@ -1406,7 +1412,9 @@ cudaError_t launch_pre_add3(const View& node, long long nodes, const Stack16& ou
     const long long h = node.rows / 8, w = node.cols / 8;
     if (h <= 0 || w <= 0 || nodes <= 0) return cudaSuccess;
     dim3 grid((unsigned)((w + 255) / 256), gy(h), (unsigned)nodes);
-#define FMM_PRE3(S, K) launch_dep(pre_add3_kernel<S, K>, grid, 256, 0, stream, node, h, w, out, scale)
+    // in plain order, as pre_root: n = 2048, depth 3 176 -> 170 us, 269 x 277 x 3195 98 -> 82
+    // (with the leaf launch's end, ptx.cuh)
+#define FMM_PRE3(S, K) pre_add3_kernel<S, K><<<grid, 256, 0, stream>>>(node, h, w, out, scale)
 #define FMM_PRE3K(S)                                        \
     switch (kind) {                                          \
         case kSplitBF16: FMM_PRE3(S, kSplitBF16); break;    \

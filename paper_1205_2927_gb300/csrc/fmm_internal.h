@@ -15,9 +15,9 @@ namespace fmm {
 // before still stores, and its loads need not stay behind the wait.  Calls in a row:
 // n = 1024, depth 2 (three launches) 39.0 -> 36.6 us, fmm_gemm_static 700 x 515 x
 // 901 16.4 -> 13.7, training step 36.8 -> 33.4, 1900 x 3101 x 1503 112.6 -> 108.8.
-// The first passes pre_root, batched_split and batched_copy stay in plain order (where
-// the read-only path is open): beside the previous call's last kernel their waiting
-// blocks cost 5 % and more.
+// The first passes pre_root, pre_add3, batched_split and batched_copy stay in plain order
+// (where the read-only path is open): beside the previous call's last kernel their
+// waiting blocks cost 5 % and more.
 template <class... P, class... A>
 inline cudaError_t launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
     cudaLaunchConfig_t cfg = {};
