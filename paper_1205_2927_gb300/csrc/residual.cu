@@ -106,7 +106,9 @@ __device__ __forceinline__ void widen(const float (&x)[N], double (&d)[N]) {
 // conversion per element of X and of v beside the FMA took 1.72 ms for the three
 // passes at 12000 x 9001 x 10500, and with the FMA alone 0.74 ms.  R = 4 on
 // 16-byte rows (four sums a row), 8 on others (one sum a row; two rows took
-// 1.6 times as long as four); below 304 blocks of that, one row per block.
+// 1.6 times as long as four); below 304 blocks of that, one row per block, off the
+// 16-byte grid with eight of its columns per thread in flight (1024 x 16001 x 1025 94 us;
+// 240 with one column at a time, 215 with a conversion per element).
 template <typename Vec, int R, bool VEC4>
 __global__ void __launch_bounds__(256, 3) rowdot64_kernel(const float* X, long long ld,
                                                                      long long rows, long long cols,
@@ -150,8 +152,31 @@ __global__ void __launch_bounds__(256, 3) rowdot64_kernel(const float* X, long l
         }
         c0 = groups << 2;
     }
+    long long c = c0 + t;
+    if constexpr (R == 1 && !VEC4) {
+        // one row: eight loads in flight come from eight of its columns (widen's branch
+        // keeps a later column's loads behind it)
+        for (; c + 7 * 256 < cols; c += 8 * 256) {
+            float q[8];
+            double d[8], w[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) q[i] = xr[0][c + 256 * i];
+            if constexpr (std::is_same<Vec, float>::value) {
+                float f[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) f[i] = v[c + 256 * i];
+                widen(f, w);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) w[i] = v[c + 256 * i];
+            }
+            widen(q, d);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) a[0][0] += d[i] * w[i];
+        }
+    }
 #pragma unroll 2
-    for (long long c = c0 + t; c < cols; c += 256) {
+    for (; c < cols; c += 256) {
         float q[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) q[r] = xr[r][c];
