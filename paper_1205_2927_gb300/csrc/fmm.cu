@@ -1587,6 +1587,21 @@ void make_child(const fmm_plan_s* p, fmm_plan_s& c) {
     }
 }
 
+// Whether a host-resident depth-0 product of less than two panels' tiles goes as two all
+// the same: half of the larger operand's and of C's transfer then hides behind a product,
+// at 205 GB/s, and while a whole product is one wave, the second panel's is another, with
+// its launches, 10 us and K steps more (by 1.3 at least: at par, 2219 x 72 x 1092 in
+// BF16x3, 98 us were 106).  Without this question: 64 x 448 x 3568 164 -> 248
+// us, 656 x 117 x 4288 236 -> 325, 1084 x 1036 x 664 105 -> 113; two panels pay for 2216 x
+// 2112 x 6607 (1.05 -> 0.89 ms).
+bool two_panels(const fmm_plan_s* c, long long K, long long tiles, long long operand, long long moved_c) {
+    if (tiles > 76) return true;
+    const double step = c->opt.precision == FMM_PREC_FP32   ? (c->pair ? 0.0175 : 0.0285)
+                        : c->opt.precision == FMM_PREC_TF32 ? (c->pair ? 0.0085 : 0.0145)
+                                                            : 0.0135;   // us per column of K, as SmallModel
+    return 0.5 * 4.0 * (double)(operand + moved_c) / 205e3 > 1.3 * (10.0 + (double)K * step);
+}
+
 // Schedules of a host-resident root: quadrants in (0..3 = 11, 12, 21, 22), sums and
 // products as soon as the quadrants before their kArrive are there, quadrants of C
 // out as soon as their products are.  With beta, C's old quadrants come in too.
@@ -1741,7 +1756,8 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
                            shares(A, p->lda, p->M, p->K, C, p->ldc, p->M, p->N) ||
                            shares(B, p->ldb, p->K, p->N, C, p->ldc, p->M, p->N);
         long long np = whole ? 1 : std::min<long long>(kHostPanels, (tiles + kPanelTiles / 2) / kPanelTiles);
-        if (np < 2) np = whole || blocks < 2 ? 1 : 2;
+        if (np < 2) np = whole || blocks < 2 || !two_panels(c, p->K, tiles, by_rows ? p->M * p->K : p->K * p->N,
+                                                             p->M * p->N * (beta != 0.0f ? 2 : 1)) ? 1 : 2;
         const long long step = (blocks + np - 1) / np * 256;   // rows or columns of a panel
         FMM_TRY(by_rows ? inB(0) : inA(0));
         int n = 0;
