@@ -1531,13 +1531,19 @@ cudaError_t launch_fill(float* p, size_t n, unsigned seed, cudaStream_t stream) 
 //    8 blocks of 1024 threads: 5250, 2365, 936     64 blocks of 256: 5360, 3055, 1160
 //   12 blocks of 1024:         5177, 2472, 948    152 blocks of 128: 5950, 3157, 1230
 //   16 blocks of 1024:         5190, 2680, 960     32 blocks of 512: 5335, 3113, 1156
+// Where little is multiplied beside the copies (a depth-0 product of less than a quarter
+// of their time), 32 blocks of 512 are ahead: 4425 x 1185 x 87 183 us, 208 with 12 of 1024;
+// 3001 x 1501 x 501 204 and 229; 2995 x 4863 x 85 440 and 510.
+// There one or two panels of C with odd rows leave the device a float per thread, the
+// whole grid at one stretch of a row (BY_GRID): 3372 x 1683 x 136 169 us, 198 by warps of
+// 512 floats; 4425 x 1185 x 87 158 and 184 (but 2995 x 4863 x 85, four panels, 512 and 440).
 // Where the products, not the copies, set the pace (the second order of a root's
-// products), 32 blocks of 512 are ahead, which with 48 registers a thread share an SM
+// products), 32 blocks of 512 are ahead as well, which with 48 registers a thread share an SM
 // with a fused leaf CTA (256 x 160 of 65536): 16384^3 29.5 ms, 32.4 with 50 registers
 // and 32.9 with 12 blocks of 1024.
 constexpr int kHostCopyBlocks = 12, kHostCopyThreads = 1024, kHostCopyBlocksWide = 32, kHostCopyThreadsWide = 512;
 constexpr int kHostCopyUnroll = 4;
-template <bool VEC>
+template <bool VEC, bool BY_GRID>
 __global__ void __maxnreg__(48) host_copy2d_kernel(const float* __restrict__ src, long long lds,
                                                           float* __restrict__ dst, long long ldd, long long rows,
                                                           long long cols) {
@@ -1562,6 +1568,12 @@ __global__ void __maxnreg__(48) host_copy2d_kernel(const float* __restrict__ src
             const long long r = i / c4, c = i - r * c4;
             reinterpret_cast<float4*>(dst + r * ldd)[c] = reinterpret_cast<const float4*>(src + r * lds)[c];
         }
+    } else if constexpr (BY_GRID) {
+        const long long total = rows * cols;
+        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
+            const long long r = i / cols, c = i - r * cols;
+            dst[r * ldd + c] = src[r * lds + c];
+        }
     } else {
         // a warp takes 512 consecutive floats of a row, sixteen loads per lane in flight
         const int lane = threadIdx.x & 31;
@@ -1582,14 +1594,15 @@ __global__ void __maxnreg__(48) host_copy2d_kernel(const float* __restrict__ src
 }
 
 cudaError_t launch_host_copy2d(const float* src, long long lds, float* dst, long long ldd, long long rows,
-                               long long cols, bool wide, cudaStream_t stream) {
+                               long long cols, bool wide, bool by_grid, cudaStream_t stream) {
     if (rows <= 0 || cols <= 0) return cudaSuccess;
     const int vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0 &&
                     lds % 4 == 0 && ldd % 4 == 0 && cols % 4 == 0;
     const unsigned blocks = wide ? kHostCopyBlocksWide : kHostCopyBlocks;
     const unsigned threads = wide ? kHostCopyThreadsWide : kHostCopyThreads;
-    if (vec) host_copy2d_kernel<true><<<blocks, threads, 0, stream>>>(src, lds, dst, ldd, rows, cols);
-    else host_copy2d_kernel<false><<<blocks, threads, 0, stream>>>(src, lds, dst, ldd, rows, cols);
+    if (vec) host_copy2d_kernel<true, false><<<blocks, threads, 0, stream>>>(src, lds, dst, ldd, rows, cols);
+    else if (by_grid) host_copy2d_kernel<false, true><<<blocks, threads, 0, stream>>>(src, lds, dst, ldd, rows, cols);
+    else host_copy2d_kernel<false, false><<<blocks, threads, 0, stream>>>(src, lds, dst, ldd, rows, cols);
     return cudaGetLastError();
 }
 

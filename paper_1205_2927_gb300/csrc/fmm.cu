@@ -1636,8 +1636,11 @@ const HostStep kOrderSlow[] = {   // P1 P2 P4 P6 P7 P5 P3
 // the rates of products of 4096 and 8192 (FP32 400 TFLOP/s), a at 205 GB/s.  First
 // and second order, ms a call (copy engines; SM copies): n = 8192 4.80, 5.02; 5.16,
 // 5.29; n = 12000 11.71, 12.00; 12.37, 12.44; n = 16384 27.7, 27.0; 30.6, 29.5.
+double host_rate(const fmm_plan_s* p) {   // of products of 4096 and 8192
+    return p->opt.precision == FMM_PREC_FP32 ? 400e12 : p->opt.precision == FMM_PREC_TF32 ? 900e12 : 600e12;
+}
 const HostStep* host_order(const fmm_plan_s* p) {
-    const double rate = p->opt.precision == FMM_PREC_FP32 ? 400e12 : p->opt.precision == FMM_PREC_TF32 ? 900e12 : 600e12;
+    const double rate = host_rate(p);
     const double c = 2.0 * (double)p->hm * (double)p->hn * (double)p->hk / rate;
     const double a = ((double)p->M * p->K + (double)p->K * p->N) * 4.0 / 8.0 / 205e9;
     return c < 1.8 * a ? kOrderFast : kOrderSlow;
@@ -1695,6 +1698,7 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
     p->host_calls += 1;
     double in_bytes = 0.0;
     const HostStep* const order = p->depth > 0 ? host_order(p) : nullptr;
+    bool wide = order == kOrderSlow, wide_out = false;   // shape of the SM copies
     fmm_plan_s* c = p->child;
     cudaEvent_t* ev = p->hev;
     float** q = p->hq;
@@ -1713,8 +1717,8 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
         if (to_dev) in_bytes += 4.0 * (double)(rows * cols);
         if (sm_copy) {
             float* hm_ = const_cast<float*>(static_cast<const float*>(host_m)) + r0 * ldh + c0;
-            if (to_dev) FMM_CUDA(launch_host_copy2d(hm_, ldh, dev, ldd, rows, cols, order == kOrderSlow, p->s_h2d));
-            else FMM_CUDA(launch_host_copy2d(dev, ldd, hm_, ldh, rows, cols, order == kOrderSlow, p->s_d2h));
+            if (to_dev) FMM_CUDA(launch_host_copy2d(hm_, ldh, dev, ldd, rows, cols, wide, false, p->s_h2d));
+            else FMM_CUDA(launch_host_copy2d(dev, ldd, hm_, ldh, rows, cols, wide, wide_out, p->s_d2h));
             p->launches += 1;
             return FMM_OK;
         }
@@ -1758,6 +1762,11 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
         long long np = whole ? 1 : std::min<long long>(kHostPanels, (tiles + kPanelTiles / 2) / kPanelTiles);
         if (np < 2) np = whole || blocks < 2 || !two_panels(c, p->K, tiles, by_rows ? p->M * p->K : p->K * p->N,
                                                              p->M * p->N * (beta != 0.0f ? 2 : 1)) ? 1 : 2;
+        const double product = 2.0 * (double)p->M * p->N * p->K / host_rate(p);
+        const double copies = 4.0 * ((double)p->M * p->K + (double)p->K * p->N + (double)p->M * p->N) / 205e9;
+        wide = product < copies / 4;   // little to multiply beside the copies
+        if (sm_copy && np > 2 && product < copies / 32) np = 1;   // next to nothing: 2995 x 4863 x 85 442 -> 388 us
+        wide_out = wide && np <= 2;
         const long long step = (blocks + np - 1) / np * 256;   // rows or columns of a panel
         FMM_TRY(by_rows ? inB(0) : inA(0));
         int n = 0;

@@ -302,6 +302,6 @@ cudaError_t launch_scale(float* C, long long ldc, long long M, long long N, floa
 // rows x cols block copy by SM loads/stores; either side may be the device
 // mapping of pinned host memory (row strides lds, ldd in elements)
 cudaError_t launch_host_copy2d(const float* src, long long lds, float* dst, long long ldd, long long rows,
-                               long long cols, bool wide, cudaStream_t stream);
+                               long long cols, bool wide, bool by_grid, cudaStream_t stream);
 
 }  // namespace fmm
