@@ -536,10 +536,12 @@ __device__ __forceinline__ void split_store(void* hi_plane, void* lo_plane, long
         if (hi_plane) __stcs(reinterpret_cast<float4*>(static_cast<float*>(hi_plane) + o), RAW ? v : h);
         // an infinity's product is its hi's alone: x - hi would be NaN
         float4 l = sub4(v, h);
-        if (isinf(v.x)) h.x = l.x = 0.f;
-        if (isinf(v.y)) h.y = l.y = 0.f;
-        if (isinf(v.z)) h.z = l.z = 0.f;
-        if (isinf(v.w)) h.w = l.w = 0.f;
+        if (isinf(fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))))) {
+            if (isinf(v.x)) h.x = l.x = 0.f;
+            if (isinf(v.y)) h.y = l.y = 0.f;
+            if (isinf(v.z)) h.z = l.z = 0.f;
+            if (isinf(v.w)) h.w = l.w = 0.f;
+        }
         uint16_t* hl = static_cast<uint16_t*>(lo_plane) + tf32x_off(o);
         __stcs(reinterpret_cast<uint2*>(hl), make_uint2(bf16x2_sat(h.x, h.y), bf16x2_sat(h.z, h.w)));
         __stcs(reinterpret_cast<uint2*>(hl + 32), make_uint2(bf16x2_sat(l.x, l.y), bf16x2_sat(l.z, l.w)));
