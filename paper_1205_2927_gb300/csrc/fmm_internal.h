@@ -13,7 +13,7 @@ namespace fmm {
 // loads: the read-only path (__ldg, const __restrict__ parameters) is for data that
 // nothing writes from a kernel's first block on, which may be resident while the kernel
 // before still stores, and its loads need not stay behind the wait.  Calls in a row:
-// n = 1024, depth 2 (three launches) 39.0 -> 36.6 us, fmm_gemm_static 700 x 515 x
+// n = 1024, depth 2 (three launches) 39.0 -> 35.5 us, fmm_gemm_static 700 x 515 x
 // 901 16.4 -> 13.7, training step 36.8 -> 33.4, 1900 x 3101 x 1503 112.6 -> 108.8.
 // The first passes pre_root, pre_add3, batched_split and batched_copy stay in plain order
 // (where the read-only path is open): beside the previous call's last kernel their
