@@ -1589,17 +1589,22 @@ void make_child(const fmm_plan_s* p, fmm_plan_s& c) {
 
 // Whether a host-resident depth-0 product of less than two panels' tiles goes as two all
 // the same: half of the larger operand's and of C's transfer then hides behind a product,
-// at 205 GB/s, and while a whole product is one wave, the second panel's is another, with
-// its launches, 10 us and K steps more (by 1.3 at least: at par, 2219 x 72 x 1092 in
-// BF16x3, 98 us were 106).  Without this question: 64 x 448 x 3568 164 -> 248
-// us, 656 x 117 x 4288 236 -> 325, 1084 x 1036 x 664 105 -> 113; two panels pay for 2216 x
-// 2112 x 6607 (1.05 -> 0.89 ms).
-bool two_panels(const fmm_plan_s* c, long long K, long long tiles, long long operand, long long moved_c) {
+// at 205 GB/s, and while a whole product is one wave, the second panel's is another, K
+// steps long, with its launches.  Copy engines take some 30 ns a row more over tight host
+// rows that are no multiple of 128 bytes (4096 rows of 1395 floats 243 us, 112 where the
+// rows lie further apart), which column panels, shorter than the rows, do not pay.  Over
+// 815 shapes of less than 96 tiles the choice loses 0.4 % to the better of one and two on
+// average (one always 3.6 %, two always 7.3 %): 64 x 448 x 3568 164 us in one, 248 in two; 656
+// x 117 x 4288 236, 325; 2216 x 2112 x 6607 1.05 ms, 0.83; 124 x 381 x 4596 BF16x3 309 us, 199.
+bool two_panels(const fmm_plan_s* p, const fmm_plan_s* c, long long tiles, bool by_rows, bool c_in, bool sm_copy) {
     if (tiles > 76) return true;
-    const double step = c->opt.precision == FMM_PREC_FP32   ? (c->pair ? 0.0175 : 0.0285)
-                        : c->opt.precision == FMM_PREC_TF32 ? (c->pair ? 0.0085 : 0.0145)
+    const double step = p->opt.precision == FMM_PREC_FP32   ? (c->pair ? 0.0175 : 0.0285)
+                        : p->opt.precision == FMM_PREC_TF32 ? (c->pair ? 0.0085 : 0.0145)
                                                             : 0.0135;   // us per column of K, as SmallModel
-    return 0.5 * 4.0 * (double)(operand + moved_c) / 205e3 > 1.3 * (10.0 + (double)K * step);
+    const double moved = (by_rows ? (double)p->M * p->K : (double)p->K * p->N) + (double)p->M * p->N * (c_in ? 2 : 1);
+    double gain = 0.5 * 4.0 * moved / 205e3;
+    if (!sm_copy && !by_rows && p->ldb - p->N < 32 && p->N % 32) gain += 0.03 * (double)(p->K + (c_in ? p->M : 0));
+    return gain > (sm_copy ? 17.0 : 10.0) + (double)p->K * step;
 }
 
 // Schedules of a host-resident root: quadrants in (0..3 = 11, 12, 21, 22), sums and
@@ -1760,8 +1765,7 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
                            shares(A, p->lda, p->M, p->K, C, p->ldc, p->M, p->N) ||
                            shares(B, p->ldb, p->K, p->N, C, p->ldc, p->M, p->N);
         long long np = whole ? 1 : std::min<long long>(kHostPanels, (tiles + kPanelTiles / 2) / kPanelTiles);
-        if (np < 2) np = whole || blocks < 2 || !two_panels(c, p->K, tiles, by_rows ? p->M * p->K : p->K * p->N,
-                                                             p->M * p->N * (beta != 0.0f ? 2 : 1)) ? 1 : 2;
+        if (np < 2) np = whole || blocks < 2 || !two_panels(p, c, tiles, by_rows, beta != 0.0f, sm_copy) ? 1 : 2;
         const double product = 2.0 * (double)p->M * p->N * p->K / host_rate(p);
         const double copies = 4.0 * ((double)p->M * p->K + (double)p->K * p->N + (double)p->M * p->N) / 205e9;
         wide = product < copies / 4;   // little to multiply beside the copies
