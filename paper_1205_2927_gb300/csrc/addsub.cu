@@ -1533,14 +1533,13 @@ cudaError_t launch_fill(float* p, size_t n, unsigned seed, cudaStream_t stream) 
 //    8 blocks of 1024 threads: 5250, 2365, 936     64 blocks of 256: 5360, 3055, 1160
 //   12 blocks of 1024:         5177, 2472, 948    152 blocks of 128: 5950, 3157, 1230
 //   16 blocks of 1024:         5190, 2680, 960     32 blocks of 512: 5335, 3113, 1156
-// Where little is multiplied beside the copies (a depth-0 product of less than a quarter
-// of their time), 32 blocks of 512 are ahead: 4425 x 1185 x 87 183 us, 208 with 12 of 1024;
-// 3001 x 1501 x 501 204 and 229; 2995 x 4863 x 85 440 and 510.
-// There one or two panels of C with odd rows leave the device a float per thread, the
-// whole grid at one stretch of a row (BY_GRID): 3372 x 1683 x 136 169 us, 198 by warps of
-// 512 floats; 4425 x 1185 x 87 158 and 184 (but 2995 x 4863 x 85, four panels, 512 and 440).
+// C of odd length and row stride, in one or two panels of a depth-0 product of less than
+// a tenth of the copies' time, leaves by 32 blocks of 512, a float per thread, the whole
+// grid at one stretch of a row (BY_GRID): 3372 x 1683 x 136 169 us, 209 by warps of 512
+// floats; 4425 x 1185 x 87 158 and 208; 3001 x 1501 x 501 185 and 229 (but 2995 x 4863 x 85 in
+// four panels 512 and 440).
 // Where the products, not the copies, set the pace (the second order of a root's
-// products), 32 blocks of 512 are ahead as well, which with 48 registers a thread share an SM
+// products), 32 blocks of 512 are ahead, which with 48 registers a thread share an SM
 // with a fused leaf CTA (256 x 160 of 65536): 16384^3 29.5 ms, 32.4 with 50 registers
 // and 32.9 with 12 blocks of 1024.
 constexpr int kHostCopyBlocks = 12, kHostCopyThreads = 1024, kHostCopyBlocksWide = 32, kHostCopyThreadsWide = 512;

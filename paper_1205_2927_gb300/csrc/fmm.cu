@@ -1703,7 +1703,8 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
     p->host_calls += 1;
     double in_bytes = 0.0;
     const HostStep* const order = p->depth > 0 ? host_order(p) : nullptr;
-    bool wide = order == kOrderSlow, wide_out = false;   // shape of the SM copies
+    const bool wide = order == kOrderSlow;   // shapes of the SM copies
+    bool odd_out = false;
     fmm_plan_s* c = p->child;
     cudaEvent_t* ev = p->hev;
     float** q = p->hq;
@@ -1723,7 +1724,7 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
         if (sm_copy) {
             float* hm_ = const_cast<float*>(static_cast<const float*>(host_m)) + r0 * ldh + c0;
             if (to_dev) FMM_CUDA(launch_host_copy2d(hm_, ldh, dev, ldd, rows, cols, wide, false, p->s_h2d));
-            else FMM_CUDA(launch_host_copy2d(dev, ldd, hm_, ldh, rows, cols, wide, wide_out, p->s_d2h));
+            else FMM_CUDA(launch_host_copy2d(dev, ldd, hm_, ldh, rows, cols, wide || odd_out, odd_out, p->s_d2h));
             p->launches += 1;
             return FMM_OK;
         }
@@ -1768,9 +1769,8 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
         if (np < 2) np = whole || blocks < 2 || !two_panels(p, c, tiles, by_rows, beta != 0.0f, sm_copy) ? 1 : 2;
         const double product = 2.0 * (double)p->M * p->N * p->K / host_rate(p);
         const double copies = 4.0 * ((double)p->M * p->K + (double)p->K * p->N + (double)p->M * p->N) / 205e9;
-        wide = product < copies / 4;   // little to multiply beside the copies
-        if (sm_copy && np > 2 && product < copies / 32) np = 1;   // next to nothing: 2995 x 4863 x 85 442 -> 388 us
-        wide_out = wide && np <= 2;
+        odd_out = sm_copy && p->ldc % 4 && p->N % 4 && product < copies / 10;
+        if (odd_out && np > 2) np = 1;   // 2995 x 4863 x 85 442 -> 388 us, 3520 x 3997 x 320 530 -> 421
         const long long step = (blocks + np - 1) / np * 256;   // rows or columns of a panel
         FMM_TRY(by_rows ? inB(0) : inA(0));
         int n = 0;
