@@ -1644,7 +1644,12 @@ const HostStep kOrderSlow[] = {   // P1 P2 P4 P6 P7 P5 P3
 double host_rate(const fmm_plan_s* p) {   // of products of 4096 and 8192
     return p->opt.precision == FMM_PREC_FP32 ? 400e12 : p->opt.precision == FMM_PREC_TF32 ? 900e12 : 600e12;
 }
-const HostStep* host_order(const fmm_plan_s* p) {
+// Where C is larger than the inputs and copy engines move it, without beta, what counts is
+// when the first quadrant of C leaves: after four of the eight input quadrants in the
+// second order, after six in the first (6000 x 6000 x 750 0.94 ms, 1.07; 6000 x 6000 x 2000
+// 1.30, 1.34; 6000 x 6000 x 3000, C as large as the inputs, 1.60, 1.56).
+const HostStep* host_order(const fmm_plan_s* p, float beta, bool sm_copy) {
+    if (!sm_copy && beta == 0.0f && (double)p->M * p->N > 1.2 * (double)p->K * (double)(p->M + p->N)) return kOrderSlow;
     const double rate = host_rate(p);
     const double c = 2.0 * (double)p->hm * (double)p->hn * (double)p->hk / rate;
     const double a = ((double)p->M * p->K + (double)p->K * p->N) * 4.0 / 8.0 / 205e9;
@@ -1702,7 +1707,7 @@ fmm_status_t run_host(fmm_plan_s* p, float alpha, const float* A, const float* B
                        p->hx_bytes[slot] <= 0.0;
     p->host_calls += 1;
     double in_bytes = 0.0;
-    const HostStep* const order = p->depth > 0 ? host_order(p) : nullptr;
+    const HostStep* const order = p->depth > 0 ? host_order(p, beta, sm_copy) : nullptr;
     const bool wide = order == kOrderSlow;   // shapes of the SM copies
     bool odd_out = false;
     fmm_plan_s* c = p->child;
