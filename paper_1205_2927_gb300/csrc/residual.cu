@@ -109,7 +109,7 @@ __device__ __forceinline__ void widen(const float (&x)[N], double (&d)[N]) {
 // 1.6 times as long as four); below 304 blocks of that, one row per block, off the
 // 16-byte grid with eight of its columns per thread in flight (1024 x 16001 x 1025 94 us;
 // 240 with one column at a time, 215 with a conversion per element).
-template <typename Vec, int R, bool VEC4>
+template <typename Vec, int R, bool VEC4, bool STEP8 = false>
 __global__ void __launch_bounds__(256, 3) rowdot64_kernel(const float* X, long long ld,
                                                                      long long rows, long long cols,
                                                                      const Vec* v,
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(256, 3) rowdot64_kernel(const float* X, long l
         c0 = groups << 2;
     }
     long long c = c0 + t;
-    if constexpr (R == 1 && !VEC4) {
+    if constexpr (STEP8) {
         // one row: eight loads in flight come from eight of its columns (widen's branch
         // keeps a later column's loads behind it)
         for (; c + 7 * 256 < cols; c += 8 * 256) {
@@ -219,6 +219,8 @@ void rowdot64(const float* X, long long ld, long long rows, long long cols, cons
         else launch_dep(rowdot64_kernel<Vec, 1, true>, grid, 256, 0, s, X, ld, rows, cols, v, out, sub);
     } else {
         if (wide) launch_dep(rowdot64_kernel<Vec, 8, false>, grid, 256, 0, s, X, ld, rows, cols, v, out, sub);
+        // shorter rows take no step of eight, and fit more blocks on an SM without it
+        else if (cols > 7 * 256) launch_dep(rowdot64_kernel<Vec, 1, false, true>, grid, 256, 0, s, X, ld, rows, cols, v, out, sub);
         else launch_dep(rowdot64_kernel<Vec, 1, false>, grid, 256, 0, s, X, ld, rows, cols, v, out, sub);
     }
 }
