@@ -876,7 +876,8 @@ __device__ __forceinline__ void split_store1(void* hi_plane, void* lo_plane, lon
 // pre_add passes.
 template <int SIDE_B, int KIND>
 __global__ void __launch_bounds__(256, 2) pre_add3_kernel(View P, long long h, long long w, Stack16 out,
-                                                       const float* scale) {
+                                                       const float* scale, int dep) {
+    if (dep) dep_start();
     const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= w) return;
     const float sc = scale ? scale[SIDE_B] : 1.0f;
@@ -1241,11 +1242,11 @@ cudaError_t launch_pre_add(const View& parent, long long nodes, const Stack& out
     const bool vec = aligned16(parent.ptr) && aligned16(out.ptr) && parent.ld % 4 == 0 && w % 4 == 0 &&
                      parent.node_stride % 4 == 0 && out.ld % 4 == 0 && out.child_stride % 4 == 0;
     dim3 grid((unsigned)((w + 4 * 128 - 1) / (4 * 128)), gy(h), (unsigned)nodes);
-    // dependent on the pass before it while a row keeps two warps busy; blocks of less work
-    // pay more for the wait than it hides (5700 x 4441 x 312, TF32, depth 3, rows of 160, 80
-    // and 40: pre-additions 74 us in plain order, 102 dependent; n = 1500, depth 2, rows of
-    // 752 and 376: 31 and 26)
-    const int dep = w >= 256;
+    // dependent on the pass before it while a row keeps two warps busy, or all blocks run at
+    // once; many blocks of less work pay more for the wait than it hides (5700 x 4441 x 312,
+    // TF32, depth 3, rows of 160, 80 and 40: pre-additions 74 us in plain order, 102 dependent;
+    // n = 1500, depth 2, rows of 752 and 376: 31 and 26; 520 x 292 x 152, depth 2, a call 24, 20)
+    const int dep = w >= 256 || (long long)grid.x * grid.y * grid.z <= 2048;
 #define FMM_PRE(V, S, F)                                                                              \
     if (dep) launch_dep(pre_add_kernel<V, S, F>, grid, 128, 0, stream, parent, h, w, out, 1);           \
     else pre_add_kernel<V, S, F><<<grid, 128, 0, stream>>>(parent, h, w, out, 0)
@@ -1414,9 +1415,13 @@ cudaError_t launch_pre_add3(const View& node, long long nodes, const Stack16& ou
     const long long h = node.rows / 8, w = node.cols / 8;
     if (h <= 0 || w <= 0 || nodes <= 0) return cudaSuccess;
     dim3 grid((unsigned)((w + 255) / 256), gy(h), (unsigned)nodes);
-    // in plain order, as pre_root: n = 2048, depth 3 176 -> 170 us, 269 x 277 x 3195 98 -> 82
-    // (with the leaf launch's end, ptx.cuh)
-#define FMM_PRE3(S, K) pre_add3_kernel<S, K><<<grid, 256, 0, stream>>>(node, h, w, out, scale)
+    // in plain order, as pre_root (n = 2048, depth 3 176 -> 170 us, 269 x 277 x 3195 98 -> 82,
+    // with the leaf launch's end, ptx.cuh), but for a handful of blocks (173 x 232 x 1220, 22
+    // of them, 63.5 -> 61.5)
+    const int dep = (long long)grid.x * grid.y * grid.z <= 24;
+#define FMM_PRE3(S, K)                                                                                      \
+    if (dep) launch_dep(pre_add3_kernel<S, K>, grid, 256, 0, stream, node, h, w, out, scale, 1);              \
+    else pre_add3_kernel<S, K><<<grid, 256, 0, stream>>>(node, h, w, out, scale, 0)
 #define FMM_PRE3K(S)                                        \
     switch (kind) {                                          \
         case kSplitBF16: FMM_PRE3(S, kSplitBF16); break;    \

@@ -736,6 +736,7 @@ fmm_status_t run_classical(fmm_plan_s* p, float alpha, const float* A, const flo
         fmm_status_t s;
         GemmGroup& G = args.groups[0];
         args.tail_shift = tail;
+        args.next_early = 1;   // the next call's splits
         args.tail_map = 4;
         if (p->pre16) {
             const size_t off = (size_t)k0 * p->es16();   // bytes; k0 is a multiple of 8

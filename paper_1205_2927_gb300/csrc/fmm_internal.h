@@ -73,6 +73,7 @@ struct GemmArgs {
     // (1 << tail_shift) of 256 rows x 256 >> tail_shift columns, through B maps of the
     // rows one CTA then stages (hi at tail_map, lo behind it)
     int tail_tiles, tail_shift, tail_map;
+    int next_early;                // a launch of one wave lets the next kernel's blocks in (ptx.cuh)
     unsigned* status;              // device status word
     // dynamic tile order of a leaf launch (null: static round robin): the next
     // free tile (zero before the launch), and one ring per CTA (per pair for

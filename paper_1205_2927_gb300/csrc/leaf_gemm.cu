@@ -280,6 +280,7 @@ __global__ void __launch_bounds__(LeafCfg<BN, MODE>::kThreads, 1) leaf_gemm_kern
                     if (++stage == Cfg::kStages) { stage = 0; phase ^= 1u; }
                 }
             }
+            if (args.next_early && total <= gridDim.x) dep_trigger();   // one wave
             if (!ok || *abort_flag) drain_fills(full_bar(0), stage, phase, issued, Cfg::kStages);
         }
     } else if (warp == 1) {
@@ -718,6 +719,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
                 }
                 }
             }
+            if (args.next_early && total <= npairs) dep_trigger();   // one wave
             // the copies of both CTAs complete on CTA 0's full barriers, and the
             // closing cluster barrier holds CTA 1 until CTA 0 has drained them
             if (rank == 0 && (!ok || *abort_flag)) drain_fills(full_bar(0), stage, phase, issued, Cfg::kStages);

@@ -32,13 +32,14 @@ __device__ __forceinline__ unsigned long long global_ns() {
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // Both, at the start of a short kernel (not of kernels of very many short blocks:
-// 350,000 blocks of a batched copy paid 5 % for the two instructions).  The persistent
-// leaf kernels do not trigger: the next kernel's blocks come when the last of theirs
-// ends.  Blocks that wait beside a leaf CTA find the SM's memory set up as its 200 KB
-// of shared memory, and the post-additions then ran on the small L1 that leaves
-// (5700 x 4441 x 312, TF32, depth 3: 479 us with a trigger behind each CTA's last tile, 426
-// without; n = 4096, depth 1 393 and 387; from a launch's start, 512 uneven products took
-// 7.22 ms, against 6.85).
+// 350,000 blocks of a batched copy paid 5 % for the two instructions).  A leaf launch of
+// one wave at depth 0, which the next call's splits follow, triggers when a block has
+// issued its tile (5688 x 172 x 684 31.3 -> 27.5 us).  Other leaf launches do not: the next
+// kernel's blocks come when the last of theirs ends.  Blocks that wait beside a leaf CTA
+// find the SM's memory set up as its 200 KB of shared memory, and the post-additions then
+// ran on the small L1 that leaves (5700 x 4441 x 312, TF32, depth 3: 479 us with a trigger
+// behind each CTA's last tile, 426 without; n = 4096, depth 1 393 and 387; n = 1024, depth 2
+// 36.7 and 35.4; from a launch's start, 512 uneven products took 7.22 ms, against 6.85).
 __device__ __forceinline__ void dep_start() {
     dep_trigger();
     dep_wait();
