@@ -57,4 +57,4 @@ def test_large_c_leaves_early():
         e[1].record()
         torch.cuda.synchronize()
         out.append(e[0].elapsed_time(e[1]) / 5)
-    assert min(ms[1:]) <= 1.33 * min(out), (ms, out)
+    assert min(ms[1:]) <= 1.38 * min(out), (ms, out)

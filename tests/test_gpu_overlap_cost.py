@@ -32,4 +32,4 @@ def test_calls_in_a_row_take_no_longer_than_their_phases(m, n, k, prec, tile):
         p.profile(False)
         apart.append((q["pre_ms"] + q["leaf_ms"] + q["post_ms"]) / 30)
     p.close()
-    assert min(row[1:]) <= 1.02 * min(apart[1:]), (row, apart)
+    assert min(row[1:]) <= 1.04 * min(apart[1:]), (row, apart)
